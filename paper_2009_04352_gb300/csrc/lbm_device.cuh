@@ -184,6 +184,27 @@ __device__ __forceinline__ float row_smag(const Phys &p, int y, int ny)
 // turns into read-only loads nor moves above the wait.
 template <typename T> constexpr bool pull_nc = std::is_same<T, float>::value;
 
+// Approximate division and square root of the collisions. The operands are
+// densities, relaxation times and stress norms, all normal numbers (or 0), for
+// which these single instructions give the bits of the full-range forms
+// (compared over every FP32 divisor from 1e-37 to 1e30); those carry scaling
+// code for subnormal and huge operands, about six instructions each, four of
+// them per cell. FULL keeps the full-range forms (the same bits).
+template <bool FULL> __device__ __forceinline__ float div_cell(float a, float b)
+{
+    if (FULL) return a / b;
+    float r;
+    asm("div.approx.ftz.f32 %0, %1, %2;" : "=f"(r) : "f"(a), "f"(b));
+    return r;
+}
+template <bool FULL> __device__ __forceinline__ float sqrt_cell(float a)
+{
+    if (FULL) return sqrtf(a);
+    float r;
+    asm("sqrt.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(a));
+    return r;
+}
+
 template <typename T> __device__ __forceinline__ float ld(const T *p);
 template <> __device__ __forceinline__ float ld<float>(const float *p) { return __ldg(p); }
 template <> __device__ __forceinline__ float ld<__half>(const __half *p) { return __half2float(__ldg(p)); }

@@ -317,10 +317,17 @@ __device__ __forceinline__ float2 mrt_odd_add(const MrtPair &m, int k, float2 dd
 // (FP32 c3: 42.3 against 41.2 GLUPS), and per step kind in the four-cell
 // kernels (quad_half). The update stores the new half values hs' = hs + de,
 // hd' = hd + dd in s and d.
+//
+// FULL keeps the full-range divisions and square roots (the same bits,
+// div_cell). The single-instruction forms measured (GLUPS, full / single) FP16
+// pull 79.1 / 81.7, MRT 67.5 / 71.5, AA 75.9 / 78.0 at 512x128x256; FP32 44.4 / 44.7;
+// FP32 MRT 42.5 / 40.5 and AA 42.7 / 41.5 by their register allocation, so those
+// two keep the full-range forms.
 template <int COLL, bool EXACT_W>
 constexpr bool PS_DEFAULT = EXACT_W != (COLL == COLL_MRT);
 
-template <int COLL = COLL_BGK, bool EXACT_W = false, bool PS = PS_DEFAULT<COLL, EXACT_W>>
+template <int COLL = COLL_BGK, bool EXACT_W = false, bool PS = PS_DEFAULT<COLL, EXACT_W>,
+          bool FULL = EXACT_W && COLL == COLL_MRT>
 __device__ __forceinline__ PairState collide_pair(float2 (&f)[Q], const Phys &p, float smag)
 {
     PairState c;
@@ -360,7 +367,7 @@ __device__ __forceinline__ PairState collide_pair(float2 (&f)[Q], const Phys &p,
     }
 
     c.rho = add2(bc(1.f), drho);
-    const float2 idev = make_float2(-drho.x / c.rho.x, -drho.y / c.rho.y);   // 1/rho - 1
+    const float2 idev = make_float2(div_cell<FULL>(-drho.x, c.rho.x), div_cell<FULL>(-drho.y, c.rho.y));   // 1/rho - 1
     if constexpr (EXACT_W) {
         // u = j + (j (1/rho - 1) + F/2 / rho), as velocity() in lbm_kernels.cuh
         c.ux = add2(jx, fma2(jx, idev, fma2(bc(p.hF[0]), idev, bc(p.hF[0]))));
@@ -392,10 +399,10 @@ __device__ __forceinline__ PairState collide_pair(float2 (&f)[Q], const Phys &p,
     float2 omega;
     {
         const float t02 = p.t02;
-        const float cqx = __fmul_rn(__fmul_rn(smag, sqrtf(q2.x)), __fadd_rn(1.f, idev.x));
-        const float cqy = __fmul_rn(__fmul_rn(smag, sqrtf(q2.y)), __fadd_rn(1.f, idev.y));
-        omega = make_float2(2.f / __fadd_rn(p.tau0, sqrtf(__fadd_rn(t02, cqx))),
-                            2.f / __fadd_rn(p.tau0, sqrtf(__fadd_rn(t02, cqy))));
+        const float cqx = __fmul_rn(__fmul_rn(smag, sqrt_cell<FULL>(q2.x)), __fadd_rn(1.f, idev.x));
+        const float cqy = __fmul_rn(__fmul_rn(smag, sqrt_cell<FULL>(q2.y)), __fadd_rn(1.f, idev.y));
+        omega = make_float2(div_cell<FULL>(2.f, __fadd_rn(p.tau0, sqrt_cell<FULL>(__fadd_rn(t02, cqx)))),
+                            div_cell<FULL>(2.f, __fadd_rn(p.tau0, sqrt_cell<FULL>(__fadd_rn(t02, cqy)))));
     }
     const float2 usq = fma2(ux, ux, fma2(uy, uy, mul2(uz, uz)));
     const float2 uF = fma2(ux, bc(p.Fx), fma2(uy, bc(p.Fy), mul2(uz, bc(p.Fz))));
@@ -602,7 +609,8 @@ __device__ __forceinline__ void pair_tile(const T *src, T *dst, const Geom &g, c
             *t = make_float4(twx.x, twz.x, twx.y, twz.y);
         }
     } else {
-        c = collide_pair<COLL, sizeof(T) == 4, LAY == LAY_PULL && PS_DEFAULT<COLL, sizeof(T) == 4>>(
+        c = collide_pair<COLL, sizeof(T) == 4, LAY == LAY_PULL && PS_DEFAULT<COLL, sizeof(T) == 4>,
+                         sizeof(T) == 4 && (COLL == COLL_MRT || LAY != LAY_PULL)>(
             f, p, row_smag(p, y, g.ny));
     }
 
