@@ -85,10 +85,12 @@ def headline_kernel(case, precision, layout=0):
 
 
 def launches_per_step(case, precision, layout=0, mrt=False):
-    """Step-kernel launches per step: the two-lattice FP16 four-cell form with
-    BGK, or with wall nodes, runs an interior-row launch and a wall-row launch
-    (with MRT and halfway walls one launch whose wall-row CTAs call a
-    separately compiled tile); every other form one."""
+    """Step-kernel launches of a step outside the library's graphs: the
+    two-lattice FP16 four-cell form with BGK, or with wall nodes, runs an
+    interior-row launch and a wall-row launch (with MRT and halfway walls one
+    launch whose wall-row CTAs call a separately compiled tile); every other form
+    one. Inside the graphs most forms run their wall rows as a launch of their
+    own, so this is a lower bound there (exact for the FP32 headline grid)."""
     from paper_2009_04352_gb300 import lbm
     quad = precision == lbm.FP16_SHIFTED and case.nx % 4 == 0
     node = case.wall == workload.WALL_WFB_NODE

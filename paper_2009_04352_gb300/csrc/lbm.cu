@@ -115,10 +115,6 @@ long long partials_per_plane(const lbm_handle *h)
     return (long long)step_grid(h).x * h->g.nz;
 }
 
-#ifndef LBM_FORK_WALL
-#define LBM_FORK_WALL 1
-#endif
-
 // Launch with programmatic stream serialisation (see pdl_begin in
 // lbm_pair.cuh) when pdl is set: the grid starts while the previous kernel on
 // the stream drains. Kernels that read the previous step's output through the
@@ -137,12 +133,6 @@ cudaError_t launch_ex(bool pdl, void (*kernel)(K...), dim3 grid, dim3 block, siz
     cfg.attrs = attr;
     cfg.numAttrs = 1;
     return cudaLaunchKernelEx(&cfg, kernel, args...);
-}
-
-template <typename... K, typename... A>
-cudaError_t launch_pdl(void (*kernel)(K...), dim3 grid, dim3 block, size_t smem, cudaStream_t s, A... args)
-{
-    return launch_ex(true, kernel, grid, block, smem, s, args...);
 }
 
 template <typename T, int NW, int COLL>
@@ -224,69 +214,150 @@ int configure_rows(lbm_handle *h)
     return rows_occupancy(h, nw, h->tma_smem, &per_sm);
 }
 
-// One step with the kernel form of the handle, collision operator COLL.
-// One in-place AA step of kind LAY (even from phase 0, odd from phase 1).
-template <int COLL, int LAY>
-cudaError_t launch_aa(lbm_handle *h, cudaStream_t s, bool stats)
+// Whether a plain step inside a graph runs as two parallel launches: the
+// interior rows, and the two wall rows as a branch of their own. Both read the
+// same source and write disjoint slots. The wall rows' CTAs are a serial chain of
+// Newton iterations several microseconds long; in one launch the last plane's
+// start last and run alone at the end of the step, and the wall layer's code
+// costs the interior rows registers. Measured (us a step, one launch / two):
+// FP32 64x32x32 5.4 / 5.4, 128x48x96 14.7 / 12.3, 256x64x128 52.4 / 50.2, AA 55.0 /
+// 51.9; FP16 MRT 256x64x128 37.3 / 32.4, 512x128x256 235.6 / 227.8, AA 256x64x128
+// 30.2 / 27.7, 64x32x32 8.6 / 5.4. The two-lattice FP32 step, bound by DRAM alone,
+// gains nothing at 512x128x256 (375.5 / 376.6) and loses 0.9% at 1024x256x512 (2961
+// / 2987), and at 64x32x32 it gains less than the larger graph costs to build, so
+// it is split between 2^18 and 2^25 cells.
+constexpr long long kSplitFp32Min = 1LL << 18, kSplitFp32Max = 1LL << 25;
+// The even AA step of the four-cell kernel is better in one launch on large
+// grids (512x128x256 step pair: 208.1 against 214.1 us a step), on small ones not
+// (256x64x128: 27.7 against 27.1, 128x48x96: 11.1 against 10.0).
+constexpr long long kWholeEvenCells = 1LL << 23;
+
+bool split_step(const lbm_handle *h)
 {
-    const dim3 grid = step_grid(h), block(h->bx);
-    void *f = h->f[0];
-    if (h->kernel == LBM_KERNEL_QUAD) {
-        __half *fh = (__half *)f;
-        // The odd step (gather and push through the neighbours, the heavier
-        // kind) calls a separately compiled wall-row tile, which frees the
-        // interior's registers (c4 FP16: 1.96 against 2.11 ms); the even step
-        // is measured faster with the wall layer inline (1.62 against 1.67 ms).
-        // Both are one launch over every row: an interior / wall-row split,
-        // as in the two-lattice step, measured slower in place.
-        if constexpr (LAY == lbm::LAY_AA_ODD)
-            if (!stats && h->g.ny > 2)
-                return launch_pdl(lbm::k_step_quad_aa_rows<false, COLL, LAY>, grid, block, 0, s, fh, h->g, h->p,
-                                  h->tw, h->part);
-        return stats ? launch_pdl(lbm::k_step_quad_aa<true, COLL, LAY>, grid, block, 0, s, fh, h->g, h->p, h->tw, h->part)
-                     : launch_pdl(lbm::k_step_quad_aa<false, COLL, LAY>, grid, block, 0, s, fh, h->g, h->p, h->tw,
-                                  h->part);
-    }
-    if (h->kernel == LBM_KERNEL_PAIR) {
-        if (h->precision == LBM_FP16_SHIFTED) {
-            __half *fh = (__half *)f;
-            return stats ? launch_pdl(lbm::k_step_pair_aa<__half, true, COLL, LAY>, grid, block, 0, s, fh, h->g, h->p,
-                                      h->tw, h->part)
-                         : launch_pdl(lbm::k_step_pair_aa<__half, false, COLL, LAY>, grid, block, 0, s, fh, h->g, h->p,
-                                      h->tw, h->part);
-        }
-        float *ff = (float *)f;
-        return stats ? launch_pdl(lbm::k_step_pair_aa<float, true, COLL, LAY>, grid, block, 0, s, ff, h->g, h->p, h->tw,
-                                  h->part)
-                     : launch_pdl(lbm::k_step_pair_aa<float, false, COLL, LAY>, grid, block, 0, s, ff, h->g, h->p,
-                                  h->tw, h->part);
-    }
-    if (h->precision == LBM_FP16_SHIFTED) {
-        if (stats)
-            lbm::k_step_aa<__half, true, COLL, LAY><<<grid, block, 0, s>>>((__half *)f, h->g, h->p, h->tw, h->part);
-        else
-            lbm::k_step_aa<__half, false, COLL, LAY><<<grid, block, 0, s>>>((__half *)f, h->g, h->p, h->tw, h->part);
-    } else {
-        if (stats)
-            lbm::k_step_aa<float, true, COLL, LAY><<<grid, block, 0, s>>>((float *)f, h->g, h->p, h->tw, h->part);
-        else
-            lbm::k_step_aa<float, false, COLL, LAY><<<grid, block, 0, s>>>((float *)f, h->g, h->p, h->tw, h->part);
-    }
-    return cudaSuccess;
+    if ((h->kernel != LBM_KERNEL_PAIR && h->kernel != LBM_KERNEL_QUAD) || h->g.ny < 3) return false;
+    const long long cells = (long long)h->g.nx * h->g.ny * h->g.nz;
+    if (h->precision == LBM_FP32 && h->layout == LBM_PULL2) return cells >= kSplitFp32Min && cells < kSplitFp32Max;
+    return true;
 }
 
+bool whole_even_step(const lbm_handle *h)
+{
+    return h->kernel == LBM_KERNEL_QUAD && (long long)h->g.nx * h->g.ny * h->g.nz >= kWholeEvenCells;
+}
+
+// The two wall rows of a step in a launch of their own, with the two-cell tile.
+template <typename T, bool STATS, int COLL, int LAY>
+cudaError_t launch_wall_rows(lbm_handle *h, cudaStream_t s, const T *src, T *dst)
+{
+    const dim3 all = step_grid(h), grid(all.x, 2, all.z);
+    const dim3 block(h->kernel == LBM_KERNEL_QUAD ? 2 * h->bx : h->bx);
+    return launch_ex(LAY != lbm::LAY_PULL || !lbm::pull_nc<T>, lbm::k_step_pair_wall<T, STATS, COLL, LAY>, grid, block, 0, s, src,
+                     dst, h->g, h->p, h->tw, h->part);
+}
+
+// The interior rows 1 .. ny - 2 of a step.
+template <typename T, bool STATS, int COLL, int LAY>
+cudaError_t launch_interior(lbm_handle *h, cudaStream_t s, const T *src, T *dst)
+{
+    const dim3 all = step_grid(h), grid(all.x, h->g.ny - 2, all.z), block(h->bx);
+    if constexpr (sizeof(T) == 2) {
+        if (h->kernel == LBM_KERNEL_QUAD) {
+            if constexpr (LAY == lbm::LAY_PULL)
+                return launch_ex(true, lbm::k_step_quad<STATS, COLL, lbm::ROWS_INTERIOR>, grid, block, 0, s, src, dst, h->g,
+                                 h->p, h->tw, h->part);
+            else
+                return launch_ex(true, lbm::k_step_quad_aa<STATS, COLL, LAY, lbm::ROWS_INTERIOR>, grid, block, 0, s, dst,
+                                 h->g, h->p, h->tw, h->part);
+        }
+    }
+    if constexpr (LAY == lbm::LAY_PULL)
+        return launch_ex(!lbm::pull_nc<T>, lbm::k_step_pair<T, STATS, COLL, lbm::ROWS_INTERIOR>, grid, block, 0, s, src, dst,
+                         h->g, h->p, h->tw, h->part);
+    else
+        return launch_ex(true, lbm::k_step_pair_aa<T, STATS, COLL, LAY, lbm::ROWS_INTERIOR>, grid, block, 0, s, dst, h->g,
+                         h->p, h->tw, h->part);
+}
+
+// A step on one stream: one launch over all rows, or the two of the BGK
+// four-cell pull step one after the other.
+template <typename T, bool STATS, int COLL, int LAY>
+cudaError_t launch_whole(lbm_handle *h, cudaStream_t s, const T *src, T *dst)
+{
+    const dim3 grid = step_grid(h), block(h->bx);
+    if (h->kernel == LBM_KERNEL_CELL) {
+        if constexpr (LAY == lbm::LAY_PULL)
+            return launch_ex(false, lbm::k_step<T, STATS, COLL>, grid, block, 0, s, src, dst, h->g, h->p, h->tw, h->part);
+        else
+            return launch_ex(false, lbm::k_step_aa<T, STATS, COLL, LAY>, grid, block, 0, s, dst, h->g, h->p, h->tw, h->part);
+    }
+    if constexpr (sizeof(T) == 2) {
+        if (h->kernel == LBM_KERNEL_QUAD) {
+            if constexpr (LAY == lbm::LAY_PULL) {
+                // BGK: the interior rows, then the two wall rows with the two-cell
+                // tile in CTAs of twice the threads; MRT: one launch whose wall-row
+                // CTAs call a separately compiled wall tile (k_step_quad_rows),
+                // which has no node form
+                if constexpr (COLL == lbm::COLL_MRT)
+                    if (h->g.ny > 2 && h->p.wall != lbm::WALL_NODE)
+                        return launch_ex(true, lbm::k_step_quad_rows<STATS, COLL>, grid, block, 0, s, src, dst, h->g, h->p, h->tw,
+                                         h->part);
+                cudaError_t e = cudaSuccess;
+                if (h->g.ny > 2) e = launch_interior<T, STATS, COLL, LAY>(h, s, src, dst);
+                return e != cudaSuccess ? e : launch_wall_rows<T, STATS, COLL, LAY>(h, s, src, dst);
+            } else {
+                // The odd step calls a separately compiled wall-row tile, which
+                // frees the interior's registers (c4 FP16: 1.96 against 2.11 ms);
+                // the even step is measured faster with the wall layer inline
+                // (1.62 against 1.67 ms).
+                if constexpr (LAY == lbm::LAY_AA_ODD && !STATS)
+                    if (h->g.ny > 2)
+                        return launch_ex(true, lbm::k_step_quad_aa_rows<STATS, COLL, LAY>, grid, block, 0, s, dst, h->g, h->p,
+                                         h->tw, h->part);
+                return launch_ex(true, lbm::k_step_quad_aa<STATS, COLL, LAY, lbm::ROWS_ALL>, grid, block, 0, s, dst, h->g,
+                                 h->p, h->tw, h->part);
+            }
+        }
+    }
+    if constexpr (LAY == lbm::LAY_PULL)
+        // read-only loads of the source lattice: no programmatic dependent launch
+        return launch_ex(!lbm::pull_nc<T>, lbm::k_step_pair<T, STATS, COLL, lbm::ROWS_ALL>, grid, block, 0, s, src, dst,
+                         h->g, h->p, h->tw, h->part);
+    else
+        return launch_ex(true, lbm::k_step_pair_aa<T, STATS, COLL, LAY, lbm::ROWS_ALL>, grid, block, 0, s, dst, h->g, h->p,
+                         h->tw, h->part);
+}
+
+// A step of layout kind LAY; s_wall non-null: the wall rows run on that stream
+// beside the interior rows.
+template <typename T, int COLL, int LAY>
+cudaError_t launch_lay(lbm_handle *h, cudaStream_t s, cudaStream_t s_wall, int src, bool stats)
+{
+    const T *a = (const T *)h->f[h->layout == LBM_AA ? 0 : src];
+    T *b = (T *)h->f[h->layout == LBM_AA ? 0 : src ^ 1];
+    if (s_wall && !(LAY == lbm::LAY_AA_EVEN && whole_even_step(h))) {
+        const cudaError_t e = launch_wall_rows<T, false, COLL, LAY>(h, s_wall, a, b);
+        if (e != cudaSuccess) return e;
+        return launch_interior<T, false, COLL, LAY>(h, s, a, b);
+    }
+    return stats ? launch_whole<T, true, COLL, LAY>(h, s, a, b) : launch_whole<T, false, COLL, LAY>(h, s, a, b);
+}
+
+template <typename T, int COLL>
+cudaError_t launch_layout(lbm_handle *h, cudaStream_t s, cudaStream_t s_wall, int src, bool stats)
+{
+    if (h->layout != LBM_AA) return launch_lay<T, COLL, lbm::LAY_PULL>(h, s, s_wall, src, stats);
+    // src is the phase: 0 runs the even step, 1 the odd step
+    return src == 0 ? launch_lay<T, COLL, lbm::LAY_AA_EVEN>(h, s, s_wall, src, stats)
+                    : launch_lay<T, COLL, lbm::LAY_AA_ODD>(h, s, s_wall, src, stats);
+}
+
+// One step with the kernel form of the handle, collision operator COLL.
 template <int COLL>
 int launch_step_c(lbm_handle *h, cudaStream_t s, int src, bool stats, cudaStream_t s_wall)
 {
-    const dim3 grid = step_grid(h), block(h->bx);
     const bool half = h->precision == LBM_FP16_SHIFTED;
-    const void *a = h->f[src];
-    void *b = h->f[src ^ 1];
     cudaError_t e = cudaSuccess;
-    if (h->layout == LBM_AA) {
-        // src is the phase: 0 runs the even step, 1 the odd step
-        e = src == 0 ? launch_aa<COLL, lbm::LAY_AA_EVEN>(h, s, stats) : launch_aa<COLL, lbm::LAY_AA_ODD>(h, s, stats);
-    } else if (h->kernel == LBM_KERNEL_TMA) {
+    if (h->kernel == LBM_KERNEL_TMA) {
         if (half) {
             if (h->tma_warps == 8)
                 launch_rows_t<__half, 8, COLL>(h, s, src, stats);
@@ -298,70 +369,10 @@ int launch_step_c(lbm_handle *h, cudaStream_t s, int src, bool stats, cudaStream
             else
                 launch_rows_t<float, 4, COLL>(h, s, src, stats);
         }
-    } else if (h->kernel == LBM_KERNEL_QUAD) {
-        // BGK: the interior rows, then the two wall rows with the two-cell tile
-        // in CTAs of twice the threads (the wall layer lives only in the second
-        // launch); MRT: one launch whose wall-row CTAs call a separately
-        // compiled wall tile (k_step_quad_rows), measured 1-2% faster for MRT
-        // and 8% slower for BGK than the two launches
-        const __half *ah = (const __half *)a;
-        __half *bh = (__half *)b;
-        bool fused = false;
-        if constexpr (COLL == lbm::COLL_MRT) {
-            fused = h->g.ny > 2 && h->p.wall != lbm::WALL_NODE;   // the called wall tile has no node form
-            if (fused)
-                e = stats ? launch_pdl(lbm::k_step_quad_rows<true, COLL>, grid, block, 0, s, ah, bh, h->g, h->p,
-                                       h->tw, h->part)
-                          : launch_pdl(lbm::k_step_quad_rows<false, COLL>, grid, block, 0, s, ah, bh, h->g, h->p,
-                                       h->tw, h->part);
-        }
-        if (!fused) {
-            // the interior rows (BGK, or MRT with wall nodes), then the wall rows
-            if (h->g.ny > 2) {
-                const dim3 gi(grid.x, h->g.ny - 2, grid.z);
-                e = stats ? launch_pdl(lbm::k_step_quad<true, COLL, lbm::ROWS_INTERIOR>, gi, block, 0, s, ah, bh,
-                                       h->g, h->p, h->tw, h->part)
-                          : launch_pdl(lbm::k_step_quad<false, COLL, lbm::ROWS_INTERIOR>, gi, block, 0, s, ah, bh,
-                                       h->g, h->p, h->tw, h->part);
-            }
-            const dim3 gw(grid.x, 2, grid.z), bw(2 * h->bx);
-            if (e == cudaSuccess)
-                e = stats ? launch_pdl(lbm::k_step_pair_wall<__half, true, COLL>, gw, bw, 0, s_wall, ah, bh, h->g,
-                                       h->p, h->tw, h->part)
-                          : launch_pdl(lbm::k_step_pair_wall<__half, false, COLL>, gw, bw, 0, s_wall, ah, bh, h->g,
-                                       h->p, h->tw, h->part);
-        }
-    } else if (h->kernel == LBM_KERNEL_PAIR) {
-        if (half) {
-            const __half *ah = (const __half *)a;
-            __half *bh = (__half *)b;
-            e = stats ? launch_pdl(lbm::k_step_pair<__half, true, COLL>, grid, block, 0, s, ah, bh, h->g, h->p, h->tw,
-                                   h->part)
-                      : launch_pdl(lbm::k_step_pair<__half, false, COLL>, grid, block, 0, s, ah, bh, h->g, h->p, h->tw,
-                                   h->part);
-        } else {
-            const float *af = (const float *)a;
-            float *bf = (float *)b;
-            // read-only loads of the source lattice: no programmatic dependent launch
-            e = stats ? launch_ex(false, lbm::k_step_pair<float, true, COLL>, grid, block, 0, s, af, bf, h->g, h->p, h->tw,
-                                   h->part)
-                      : launch_ex(false, lbm::k_step_pair<float, false, COLL>, grid, block, 0, s, af, bf, h->g, h->p, h->tw,
-                                   h->part);
-        }
     } else if (half) {
-        if (stats)
-            lbm::k_step<__half, true, COLL><<<grid, block, 0, s>>>((const __half *)a, (__half *)b, h->g, h->p, h->tw,
-                                                                   h->part);
-        else
-            lbm::k_step<__half, false, COLL><<<grid, block, 0, s>>>((const __half *)a, (__half *)b, h->g, h->p, h->tw,
-                                                                    h->part);
+        e = launch_layout<__half, COLL>(h, s, s_wall, src, stats);
     } else {
-        if (stats)
-            lbm::k_step<float, true, COLL><<<grid, block, 0, s>>>((const float *)a, (float *)b, h->g, h->p, h->tw,
-                                                                  h->part);
-        else
-            lbm::k_step<float, false, COLL><<<grid, block, 0, s>>>((const float *)a, (float *)b, h->g, h->p, h->tw,
-                                                                   h->part);
+        e = launch_layout<float, COLL>(h, s, s_wall, src, stats);
     }
     if (e != cudaSuccess) return fail(LBM_ERR_CUDA, "step launch: %s", cudaGetErrorString(e));
     CK_LAUNCH();
@@ -374,23 +385,12 @@ int launch_step_c(lbm_handle *h, cudaStream_t s, int src, bool stats, cudaStream
     return LBM_OK;
 }
 
-// One step on stream s; the wall-row launch of a two-launch four-cell step goes
-// to s_wall (s when null).
+// One step on stream s; with s_wall a plain step's wall rows go to that stream
+// as a launch of their own (split_step).
 int launch_step(lbm_handle *h, cudaStream_t s, int src, bool stats, cudaStream_t s_wall = nullptr)
 {
-    if (!s_wall) s_wall = s;
     return h->p.collision == lbm::COLL_MRT ? launch_step_c<lbm::COLL_MRT>(h, s, src, stats, s_wall)
                                            : launch_step_c<lbm::COLL_BGK>(h, s, src, stats, s_wall);
-}
-
-// Whether a plain step is the two-launch four-cell form (interior rows, then
-// the wall rows with the two-cell tile): both read the source lattice and
-// write disjoint rows of the destination, so inside a graph the wall-row
-// launch is a parallel branch of the step instead of running after it.
-bool two_launch_step(const lbm_handle *h)
-{
-    return h->kernel == LBM_KERNEL_QUAD && h->layout == LBM_PULL2 && h->g.ny > 2 &&
-           (h->p.collision == lbm::COLL_BGK || h->p.wall == lbm::WALL_NODE);
 }
 
 int build_chunk(lbm_handle *h, int start)
@@ -398,7 +398,7 @@ int build_chunk(lbm_handle *h, int start)
     cudaGraph_t graph = nullptr;
     CK(cudaStreamBeginCapture(h->cap, cudaStreamCaptureModeThreadLocal));
     int rc = LBM_OK;
-    const bool fork = LBM_FORK_WALL && two_launch_step(h);
+    const bool fork = split_step(h);
     cudaError_t ce = cudaSuccess;
     for (int i = 0; i < kGraphSteps && rc == LBM_OK && ce == cudaSuccess; ++i) {
         if (fork) {

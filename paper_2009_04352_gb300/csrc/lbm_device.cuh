@@ -295,6 +295,16 @@ __device__ __forceinline__ long long push_offset(const Geom &g, int wall, int a,
     return (long long)slot * g.plane + ((long long)zt * g.ny + yt) * g.sx + xt;
 }
 
+// Row (y, z) of a step kernel's block.
+enum { ROWS_ALL = 0, ROWS_INTERIOR = 1, ROWS_WALL = 2 };
+template <int ROWS>
+__device__ __forceinline__ void row_of_block(const Geom &g, int &y, int &z)
+{
+    z = blockIdx.z;
+    y = ROWS == ROWS_INTERIOR ? (int)blockIdx.y + 1
+                              : (ROWS == ROWS_WALL ? (blockIdx.y == 0 ? 0 : g.ny - 1) : (int)blockIdx.y);
+}
+
 struct Nbr {
     int xm, xp, zm, zp;
 };
@@ -437,12 +447,44 @@ __device__ __forceinline__ float powerlaw_uplus(float R, const Phys &p)
     return R <= p.law_r2 ? r2 : p.pw_a * sqrtf(sqrtf(r2));
 }
 
+// One Newton step of Spalding's law for a lane: u+ and whether it has stopped.
+__device__ __forceinline__ void spalding_step(float R, const Phys &p, float &up, bool &done)
+{
+    const float k = p.kappa * up;
+    const float ek = expf(k);
+    const float k2 = __fmul_rn(k, k);
+    const float t2 = __fsub_rn(__fsub_rn(__fsub_rn(ek, 1.f), k), __fmul_rn(0.5f, k2));   // e^k - 1 - k - k^2/2
+    const float t3 = __fsub_rn(t2, __fmul_rn(__fmul_rn(k2, k), 1.f / 6.f));            // ... - k^3/6
+    const float S = __fmaf_rn(p.ekb, t3, up);                                           // y+(u+)
+    const float dS = __fmaf_rn(__fmul_rn(p.ekb, p.kappa), t2, 1.f);                     // dy+/du+
+    const float step = done ? 0.f : div_cell<false>(__fmaf_rn(up, S, -R), __fmaf_rn(up, dS, S));
+    up -= step;
+    done = done || fabsf(step) <= 1e-7f * up;
+}
+
 // u+ of the selected wall function (p.law is uniform over the launch).
 __device__ __forceinline__ float wall_uplus(float R, const Phys &p, unsigned mask)
 {
     if (p.law == LAW_LOG) return loglaw_uplus(R, p, mask);
     if (p.law == LAW_POWER) return powerlaw_uplus(R, p);
     return spalding_uplus(R, p, mask);
+}
+
+// u+ of the selected wall function for two cells of a thread at once.
+__device__ __forceinline__ float2 wall_uplus2(float2 R, const Phys &p, unsigned mask)
+{
+    if (p.law == LAW_LOG) return make_float2(loglaw_uplus(R.x, p, mask), loglaw_uplus(R.y, p, mask));
+    if (p.law == LAW_POWER) return make_float2(powerlaw_uplus(R.x, p), powerlaw_uplus(R.y, p));
+    float2 up = make_float2(sqrtf(R.x), sqrtf(R.y));
+    if (R.x > 100.f) up.x = fminf(up.x, __fadd_rn(logf(R.x) / p.kappa, p.B));
+    if (R.y > 100.f) up.y = fminf(up.y, __fadd_rn(logf(R.y) / p.kappa, p.B));
+    bool d0 = false, d1 = false;
+    for (int it = 0; it < p.newton_iters; ++it) {
+        spalding_step(R.x, p, up.x, d0);
+        spalding_step(R.y, p, up.y, d1);
+        if (__all_sync(mask, d0 && d1)) break;
+    }
+    return up;
 }
 
 }  // namespace lbm

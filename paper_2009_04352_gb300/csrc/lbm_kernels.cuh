@@ -199,6 +199,28 @@ __device__ __forceinline__ void wfb_stress(const CellState &c, const Phys &p, un
     }
 }
 
+// wfb_stress for two cells of a thread (c and b), their wall laws solved together.
+__device__ __forceinline__ void wfb_stress2(const CellState &c, const CellState &b, const Phys &p, float2 &twx,
+                                            float2 &twz)
+{
+    twx = make_float2(0.f, 0.f);
+    twz = make_float2(0.f, 0.f);
+    const float ut = sqrtf(__fmaf_rn(c.uz, c.uz, __fmul_rn(c.ux, c.ux)));
+    const float vt = sqrtf(__fmaf_rn(b.uz, b.uz, __fmul_rn(b.ux, b.ux)));
+    const float2 up = wall_uplus2(make_float2(fmaxf(p.y1_over_nu * ut, 1e-30f), fmaxf(p.y1_over_nu * vt, 1e-30f)), p,
+                                  0xffffffffu);
+    const float us = ut / up.x, vs = vt / up.y;
+    const float tu = c.rho * us * us, tv = b.rho * vs * vs;
+    if (ut > 0.f) {
+        twx.x = -c.ux / ut * tu;
+        twz.x = -c.uz / ut * tu;
+    }
+    if (vt > 0.f) {
+        twx.y = -b.ux / vt * tv;
+        twz.y = -b.uz / vt * tv;
+    }
+}
+
 // Full-way WFB at a wall node (layer 0 or ny - 1, WALL_NODE): f holds the
 // node's gathered populations and ca the state of the first fluid node. fs
 // receives what the node sends out: for each population b entering the fluid
@@ -378,7 +400,8 @@ __device__ __forceinline__ void cell_step(const T *src, T *dst, const Geom &g, c
                                           double *part)
 {
     const int x = blockIdx.x * blockDim.x + threadIdx.x;
-    const int y = blockIdx.y, z = blockIdx.z;
+    int y, z;
+    row_of_block<ROWS_ALL>(g, y, z);
     const bool valid = x < g.nx;
     if (!STATS && !valid) return;
     const int xc = valid ? x : 0;
@@ -456,7 +479,7 @@ __device__ __forceinline__ void cell_step(const T *src, T *dst, const Geom &g, c
     }
 }
 
-template <typename T, bool STATS, int COLL = COLL_BGK>
+template <typename T, bool STATS, int COLL>
 __global__ void __launch_bounds__(128) k_step(const T *__restrict__ src, T *__restrict__ dst, Geom g, Phys p,
                                               float *__restrict__ tw_out, double *__restrict__ part)
 {

@@ -193,8 +193,7 @@ __device__ __forceinline__ void wall_layer_pair(float2 (&f)[Q], const PairState 
     twz = make_float2(0.f, 0.f);
     if (p.wall == WALL_WFB) {
         const CellState ca{c.rho.x, c.ux.x, c.uy.x, c.uz.x}, cb{c.rho.y, c.ux.y, c.uy.y, c.uz.y};
-        wfb_stress(ca, p, 0xffffffffu, twx.x, twz.x);
-        wfb_stress(cb, p, 0xffffffffu, twx.y, twz.y);
+        wfb_stress2(ca, cb, p, twx, twz);
         const float2 hx = make_float2(0.5f * twx.x, 0.5f * twx.y), hz = make_float2(0.5f * twz.x, 0.5f * twz.y);
         const float2 mhx = make_float2(-hx.x, -hx.y), mhz = make_float2(-hz.x, -hz.y);
         if (bottom) {
@@ -320,9 +319,8 @@ __device__ __forceinline__ float2 mrt_odd_add(const MrtPair &m, int k, float2 dd
 //
 // FULL keeps the full-range divisions and square roots (the same bits,
 // div_cell). The single-instruction forms measured (GLUPS, full / single) FP16
-// pull 79.1 / 81.7, MRT 67.5 / 71.5, AA 75.9 / 78.0 at 512x128x256; FP32 44.4 / 44.7;
-// FP32 MRT 42.5 / 40.5 and AA 42.7 / 41.5 by their register allocation, so those
-// two keep the full-range forms.
+// pull 79.1 / 81.7, MRT 67.5 / 71.5, AA 75.9 / 78.0 at 512x128x256, FP32 44.4 / 44.7;
+// FP32 MRT, by its register allocation, 42.3 / 41.5, so it keeps the full range.
 template <int COLL, bool EXACT_W>
 constexpr bool PS_DEFAULT = EXACT_W != (COLL == COLL_MRT);
 
@@ -543,10 +541,7 @@ __device__ __forceinline__ PairState collide_pair(float2 (&f)[Q], const Phys &p,
 //
 // LAY selects the storage scheme (LAY_PULL: src and dst are the two lattices;
 // LAY_AA_EVEN / LAY_AA_ODD: src == dst, the single AA array).
-// Row sets a tile instantiation serves: any row, the interior rows only (no
-// wall-layer code in the instantiation), or the two wall rows only.
-enum { ROWS_ALL = 0, ROWS_INTERIOR = 1, ROWS_WALL = 2 };
-
+// ROWS: the row set the instantiation serves (no wall-layer code for the interior rows).
 template <typename T, bool STATS, int COLL = COLL_BGK, int LAY = LAY_PULL, int ROWS = ROWS_ALL>
 __device__ __forceinline__ void pair_tile(const T *src, T *dst, const Geom &g, const Phys &p,
                                           float *__restrict__ tw_out, double *__restrict__ part_blk, int xb, int y,
@@ -609,24 +604,12 @@ __device__ __forceinline__ void pair_tile(const T *src, T *dst, const Geom &g, c
             *t = make_float4(twx.x, twz.x, twx.y, twz.y);
         }
     } else {
-        c = collide_pair<COLL, sizeof(T) == 4, LAY == LAY_PULL && PS_DEFAULT<COLL, sizeof(T) == 4>,
-                         sizeof(T) == 4 && (COLL == COLL_MRT || LAY != LAY_PULL)>(
+        c = collide_pair<COLL, sizeof(T) == 4, LAY == LAY_PULL && PS_DEFAULT<COLL, sizeof(T) == 4>>(
             f, p, row_smag(p, y, g.ny));
     }
 
     if (ROWS != ROWS_INTERIOR && !node_row && (y == 0 || y == g.ny - 1)) {
-        // the wall layer of both cells, lane by lane (all 32 lanes are present)
-        float fa[Q], fb[Q];
-#pragma unroll
-        for (int a = 0; a < Q; ++a) {
-            fa[a] = f[a].x;
-            fb[a] = f[a].y;
-        }
-        const CellState ca{c.rho.x, c.ux.x, c.uy.x, c.uz.x}, cb{c.rho.y, c.ux.y, c.uy.y, c.uz.y};
-        wall_layer(fa, ca, p, y == 0, 0xffffffffu, twx.x, twz.x);
-        wall_layer(fb, cb, p, y == 0, 0xffffffffu, twx.y, twz.y);
-#pragma unroll
-        for (int a = 0; a < Q; ++a) f[a] = make_float2(fa[a], fb[a]);
+        wall_layer_pair(f, c, p, y == 0, twx, twz);   // all 32 lanes are present
         if (valid) {
             float4 *t = reinterpret_cast<float4 *>(
                 reinterpret_cast<float2 *>(tw_out) + ((long long)((y == 0 ? 0 : 1) * g.nz + z) * g.nx + x0));
@@ -634,9 +617,9 @@ __device__ __forceinline__ void pair_tile(const T *src, T *dst, const Geom &g, c
         }
     }
     if (LAY == LAY_AA_ODD) {
-        if (y == 0)
+        if (ROWS != ROWS_INTERIOR && y == 0)
             push_pair<T, ROW_BOTTOM>(dst, g, p.wall, xl, y, z, zm, zp, lane, valid, f);
-        else if (y == g.ny - 1)
+        else if (ROWS != ROWS_INTERIOR && y == g.ny - 1)
             push_pair<T, ROW_TOP>(dst, g, p.wall, xl, y, z, zm, zp, lane, valid, f);
         else
             push_pair<T, ROW_INTERIOR>(dst, g, p.wall, xl, y, z, zm, zp, lane, valid, f);
@@ -680,44 +663,47 @@ __device__ __forceinline__ void pdl_begin()
 #define LBM_PAIR_MRT_MIN_BLOCKS 5   // the same for the MRT instantiations (96 registers)
 #endif
 
-template <typename T, bool STATS, int COLL = COLL_BGK>
-__global__ void __launch_bounds__(128, COLL == COLL_MRT ? LBM_PAIR_MRT_MIN_BLOCKS : LBM_PAIR_MIN_BLOCKS) k_step_pair(const T *__restrict__ src, T *__restrict__ dst, Geom g, Phys p,
-                                                   float *__restrict__ tw_out, double *__restrict__ part)
+template <typename T, bool STATS, int COLL, int ROWS>
+__global__ void __launch_bounds__(128, COLL == COLL_MRT ? LBM_PAIR_MRT_MIN_BLOCKS : LBM_PAIR_MIN_BLOCKS)
+    k_step_pair(const T *__restrict__ src, T *__restrict__ dst, Geom g, Phys p, float *__restrict__ tw_out,
+                double *__restrict__ part)
 {
     pdl_begin();
-    const int y = blockIdx.y, z = blockIdx.z;
+    int y, z;
+    row_of_block<ROWS>(g, y, z);
     const long long blk = ((long long)y * g.nz + z) * gridDim.x + blockIdx.x;
-    pair_tile<T, STATS, COLL>(src, dst, g, p, tw_out, STATS ? part + blk * K_PART : nullptr, blockIdx.x, y, z);
+    pair_tile<T, STATS, COLL, LAY_PULL, ROWS>(src, dst, g, p, tw_out, STATS ? part + blk * K_PART : nullptr, blockIdx.x,
+                                              y, z);
 }
 
-// The two wall rows of the four-cell (FP16) step, run with the two-cell tile:
-// a CTA of twice the four-cell launch's threads covers the same cells as one
-// four-cell CTA (so the partial sums keep the four-cell layout) and each
-// thread carries half the serial work (wall law, collision) of a four-cell
-// thread, which shortens this one-wave, latency-bound launch. The two tile
-// forms compute the same bits. grid (four-cell tiles per row, 2, nz); LAY as
-// in pair_tile (for the AA kinds src == dst).
+// The two wall rows of a step whose interior rows run in a launch of their
+// own, with the two-cell tile. Beside the four-cell interior a CTA has twice the
+// interior launch's threads, so that it covers the same cells (the partial sums
+// keep that layout) and each thread carries half the serial work (wall law,
+// collision) of a four-cell thread; the two tile forms compute the same bits.
+// grid (tiles per row, 2, nz); LAY as in pair_tile (for the AA kinds src == dst).
 template <typename T, bool STATS, int COLL, int LAY = LAY_PULL>
 __global__ void __launch_bounds__(256) k_step_pair_wall(const T *src, T *dst, Geom g, Phys p,
                                                         float *__restrict__ tw_out, double *__restrict__ part)
 {
     pdl_begin();
-    const int y = blockIdx.y == 0 ? 0 : g.ny - 1, z = blockIdx.z;
+    int y, z;
+    row_of_block<ROWS_WALL>(g, y, z);
     const long long blk = ((long long)y * g.nz + z) * gridDim.x + blockIdx.x;
     pair_tile<T, STATS, COLL, LAY, ROWS_WALL>(src, dst, g, p, tw_out, STATS ? part + blk * K_PART : nullptr,
                                               blockIdx.x, y, z);
 }
 
 // The two-cell step on the single AA array (LAY_AA_EVEN or LAY_AA_ODD).
-template <typename T, bool STATS, int COLL, int LAY>
-__global__ void __launch_bounds__(128, COLL == COLL_MRT ? LBM_PAIR_MRT_MIN_BLOCKS : LBM_PAIR_MIN_BLOCKS) k_step_pair_aa(T *f, Geom g, Phys p,
-                                                                            float *__restrict__ tw_out,
-                                                                            double *__restrict__ part)
+template <typename T, bool STATS, int COLL, int LAY, int ROWS>
+__global__ void __launch_bounds__(128, COLL == COLL_MRT ? LBM_PAIR_MRT_MIN_BLOCKS : LBM_PAIR_MIN_BLOCKS)
+    k_step_pair_aa(T *f, Geom g, Phys p, float *__restrict__ tw_out, double *__restrict__ part)
 {
     pdl_begin();
-    const int y = blockIdx.y, z = blockIdx.z;
+    int y, z;
+    row_of_block<ROWS>(g, y, z);
     const long long blk = ((long long)y * g.nz + z) * gridDim.x + blockIdx.x;
-    pair_tile<T, STATS, COLL, LAY>(f, f, g, p, tw_out, STATS ? part + blk * K_PART : nullptr, blockIdx.x, y, z);
+    pair_tile<T, STATS, COLL, LAY, ROWS>(f, f, g, p, tw_out, STATS ? part + blk * K_PART : nullptr, blockIdx.x, y, z);
 }
 
 }  // namespace lbm

@@ -240,7 +240,7 @@ __device__ __forceinline__ void quad_half(uint2 (&r)[Q], const Phys &p, float sm
 
 // Collision, wall layer, store (or AA push) and statistics of the quad whose
 // 19 populations the gather left in r (the part of a tile after its loads).
-template <bool STATS, int COLL, int LAY, int ROWS>
+template <bool STATS, int COLL, int LAY, int ROWS, bool HIDE>
 __device__ __forceinline__ void quad_finish(uint2 (&r)[Q], __half *dst, const Geom &g, const Phys &p,
                                             float *__restrict__ tw_out, double *__restrict__ part_blk, int x0, int xl,
                                             bool valid, int y, int z, int zm, int zp, int lane)
@@ -259,6 +259,11 @@ __device__ __forceinline__ void quad_finish(uint2 (&r)[Q], __half *dst, const Ge
         t[1] = twb;
     }
     if (LAY == LAY_AA_ODD) {
+        // the push targets are the gather's sources (slot a of x + e_a is what
+        // direction opp(a) read): with HIDE the row indices are made opaque here,
+        // or the 19 addresses stay live through the collision (152 B of spills a
+        // thread in the interior-only kernel against 28 B)
+        if (HIDE) asm volatile("" : "+r"(y), "+r"(z), "+r"(zm), "+r"(zp));
         if (ROWS != ROWS_INTERIOR && y == 0)
             push_quad<ROW_BOTTOM>(dst, g, p.wall, xl, y, z, zm, zp, lane, valid, r);
         else if (ROWS != ROWS_INTERIOR && y == g.ny - 1)
@@ -274,7 +279,7 @@ __device__ __forceinline__ void quad_finish(uint2 (&r)[Q], __half *dst, const Ge
     if (STATS) stats_block_store(v, part_blk);
 }
 
-template <bool STATS, int COLL = COLL_BGK, int LAY = LAY_PULL, int ROWS = ROWS_ALL>
+template <bool STATS, int COLL = COLL_BGK, int LAY = LAY_PULL, int ROWS = ROWS_ALL, bool HIDE = false>
 __device__ __forceinline__ void quad_tile(const __half *src, __half *dst, const Geom &g, const Phys &p,
                                           float *__restrict__ tw_out, double *__restrict__ part_blk, int xb, int y,
                                           int z)
@@ -292,14 +297,14 @@ __device__ __forceinline__ void quad_tile(const __half *src, __half *dst, const 
         gather_quad<ROW_TOP, LAY>(src, g, p.wall, xl, y, z, zm, zp, lane, r);
     else
         gather_quad<ROW_INTERIOR, LAY>(src, g, p.wall, xl, y, z, zm, zp, lane, r);
-    quad_finish<STATS, COLL, LAY, ROWS>(r, dst, g, p, tw_out, part_blk, x0, xl, valid, y, z, zm, zp, lane);
+    quad_finish<STATS, COLL, LAY, ROWS, HIDE>(r, dst, g, p, tw_out, part_blk, x0, xl, valid, y, z, zm, zp, lane);
 }
 
 // The two-lattice step over the row set ROWS: grid.y is ny (ROWS_ALL), ny - 2
 // (ROWS_INTERIOR, row blockIdx.y + 1) or 2 (ROWS_WALL, rows 0 and ny - 1).
 // The step runs as an interior launch and a wall-row launch, so that the wall
 // layer's code does not shape the register allocation of the interior rows.
-template <bool STATS, int COLL = COLL_BGK, int ROWS = ROWS_ALL>
+template <bool STATS, int COLL, int ROWS>
 __global__ void __launch_bounds__(128, COLL == COLL_MRT ? LBM_QUAD_MRT_MIN_BLOCKS
                                                          : (STATS ? LBM_QUAD_STATS_MIN_BLOCKS : LBM_QUAD_MIN_BLOCKS))
     k_step_quad(const __half *__restrict__ src,
@@ -308,9 +313,8 @@ __global__ void __launch_bounds__(128, COLL == COLL_MRT ? LBM_QUAD_MRT_MIN_BLOCK
                                                                          double *__restrict__ part)
 {
     pdl_begin();
-    const int y = ROWS == ROWS_INTERIOR ? (int)blockIdx.y + 1
-                                        : (ROWS == ROWS_WALL ? (blockIdx.y == 0 ? 0 : g.ny - 1) : (int)blockIdx.y);
-    const int z = blockIdx.z;
+    int y, z;
+    row_of_block<ROWS>(g, y, z);
     const long long blk = ((long long)y * g.nz + z) * gridDim.x + blockIdx.x;
     quad_tile<STATS, COLL, LAY_PULL, ROWS>(src, dst, g, p, tw_out, STATS ? part + blk * K_PART : nullptr,
                                            blockIdx.x, y, z);
@@ -337,7 +341,8 @@ __global__ void __launch_bounds__(128, COLL == COLL_MRT ? LBM_QUAD_MRT_MIN_BLOCK
                      float *__restrict__ tw_out, double *__restrict__ part)
 {
     pdl_begin();
-    const int y = blockIdx.y, z = blockIdx.z;
+    int y, z;
+    row_of_block<ROWS_ALL>(g, y, z);
     const long long blk = ((long long)y * g.nz + z) * gridDim.x + blockIdx.x;
     double *pb = STATS ? part + blk * K_PART : nullptr;
     if (y == 0 || y == g.ny - 1)
@@ -349,7 +354,7 @@ __global__ void __launch_bounds__(128, COLL == COLL_MRT ? LBM_QUAD_MRT_MIN_BLOCK
 // The four-cell step on the single AA array (LAY_AA_EVEN or LAY_AA_ODD) over
 // the row set ROWS (grid.y ny, or ny - 2 for the interior rows, row
 // blockIdx.y + 1).
-template <bool STATS, int COLL, int LAY, int ROWS = ROWS_ALL>
+template <bool STATS, int COLL, int LAY, int ROWS>
 __global__ void __launch_bounds__(128, COLL == COLL_MRT ? LBM_QUAD_MRT_MIN_BLOCKS
                                                          : (STATS ? LBM_QUAD_STATS_MIN_BLOCKS : LBM_QUAD_AA_MIN_BLOCKS))
     k_step_quad_aa(__half *f, Geom g, Phys p,
@@ -357,9 +362,10 @@ __global__ void __launch_bounds__(128, COLL == COLL_MRT ? LBM_QUAD_MRT_MIN_BLOCK
                                                                             double *__restrict__ part)
 {
     pdl_begin();
-    const int y = ROWS == ROWS_INTERIOR ? (int)blockIdx.y + 1 : (int)blockIdx.y, z = blockIdx.z;
+    int y, z;
+    row_of_block<ROWS>(g, y, z);
     const long long blk = ((long long)y * g.nz + z) * gridDim.x + blockIdx.x;
-    quad_tile<STATS, COLL, LAY, ROWS>(f, f, g, p, tw_out, STATS ? part + blk * K_PART : nullptr, blockIdx.x, y, z);
+    quad_tile<STATS, COLL, LAY, ROWS, ROWS == ROWS_INTERIOR>(f, f, g, p, tw_out, STATS ? part + blk * K_PART : nullptr, blockIdx.x, y, z);
 }
 
 // The wall-row tile of the four-cell AA step, compiled apart from the
@@ -379,7 +385,8 @@ __global__ void __launch_bounds__(128, LBM_QUAD_AA_ROWS_MIN_BLOCKS)
     k_step_quad_aa_rows(__half *f, Geom g, Phys p, float *__restrict__ tw_out, double *__restrict__ part)
 {
     pdl_begin();
-    const int y = blockIdx.y, z = blockIdx.z;
+    int y, z;
+    row_of_block<ROWS_ALL>(g, y, z);
     const long long blk = ((long long)y * g.nz + z) * gridDim.x + blockIdx.x;
     double *pb = STATS ? part + blk * K_PART : nullptr;
     if (y == 0 || y == g.ny - 1)
