@@ -80,6 +80,18 @@ int select_kernel(lbm_handle *h, int kernel)
     h->kernel = kernel;
     const int per_row = h->g.nx / cells_per_thread(kernel);
     h->bx = per_row >= 128 ? 128 : (per_row > 32 ? 64 : 32);   // <= the kernels' launch bound of 128
+    // Steps from lattice (or phase) 1 walk the planes backwards, so that each
+    // step begins with the planes the step before wrote last, which L2 still
+    // holds. Measured (us a step, forwards only / alternating): FP32 256x64x128
+    // (319 MB) 50.2 / 47.7, AA (159 MB) 51.9 / 43.1, 512x128x256 AA 390 / 380, FP16
+    // 256x64x128 29.4 / 28.6. Lattices that stay in L2 as a whole gain nothing and
+    // lose the near half of the two-die L2 (128x48x96 FP32, 90 MB: 12.3 / 12.8), so
+    // the line is three quarters of L2.
+    int dev = 0, l2 = 0;
+    CK(cudaGetDevice(&dev));
+    CK(cudaDeviceGetAttribute(&l2, cudaDevAttrL2CacheSize, dev));
+    const size_t lattices = (size_t)(h->layout == LBM_AA ? 1 : 2) * lbm::Q * h->g.plane * elem_size(h);
+    h->reverse = lattices >= (size_t)l2 / 4 * 3;
     if (kernel == LBM_KERNEL_TMA) {
         const int rc = configure_rows(h);
         if (rc != LBM_OK) return rc;
@@ -256,25 +268,25 @@ cudaError_t launch_wall_rows(lbm_handle *h, cudaStream_t s, const T *src, T *dst
 }
 
 // The interior rows 1 .. ny - 2 of a step.
-template <typename T, bool STATS, int COLL, int LAY>
+template <typename T, bool STATS, int COLL, int LAY, bool REV>
 cudaError_t launch_interior(lbm_handle *h, cudaStream_t s, const T *src, T *dst)
 {
     const dim3 all = step_grid(h), grid(all.x, h->g.ny - 2, all.z), block(h->bx);
     if constexpr (sizeof(T) == 2) {
         if (h->kernel == LBM_KERNEL_QUAD) {
             if constexpr (LAY == lbm::LAY_PULL)
-                return launch_ex(true, lbm::k_step_quad<STATS, COLL, lbm::ROWS_INTERIOR>, grid, block, 0, s, src, dst, h->g,
+                return launch_ex(true, lbm::k_step_quad<STATS, COLL, lbm::ROWS_INTERIOR, REV>, grid, block, 0, s, src, dst, h->g,
                                  h->p, h->tw, h->part);
             else
-                return launch_ex(true, lbm::k_step_quad_aa<STATS, COLL, LAY, lbm::ROWS_INTERIOR>, grid, block, 0, s, dst,
+                return launch_ex(true, lbm::k_step_quad_aa<STATS, COLL, LAY, lbm::ROWS_INTERIOR, REV>, grid, block, 0, s, dst,
                                  h->g, h->p, h->tw, h->part);
         }
     }
     if constexpr (LAY == lbm::LAY_PULL)
-        return launch_ex(!lbm::pull_nc<T>, lbm::k_step_pair<T, STATS, COLL, lbm::ROWS_INTERIOR>, grid, block, 0, s, src, dst,
+        return launch_ex(!lbm::pull_nc<T>, lbm::k_step_pair<T, STATS, COLL, lbm::ROWS_INTERIOR, REV>, grid, block, 0, s, src, dst,
                          h->g, h->p, h->tw, h->part);
     else
-        return launch_ex(true, lbm::k_step_pair_aa<T, STATS, COLL, LAY, lbm::ROWS_INTERIOR>, grid, block, 0, s, dst, h->g,
+        return launch_ex(true, lbm::k_step_pair_aa<T, STATS, COLL, LAY, lbm::ROWS_INTERIOR, REV>, grid, block, 0, s, dst, h->g,
                          h->p, h->tw, h->part);
 }
 
@@ -302,7 +314,7 @@ cudaError_t launch_whole(lbm_handle *h, cudaStream_t s, const T *src, T *dst)
                         return launch_ex(true, lbm::k_step_quad_rows<STATS, COLL>, grid, block, 0, s, src, dst, h->g, h->p, h->tw,
                                          h->part);
                 cudaError_t e = cudaSuccess;
-                if (h->g.ny > 2) e = launch_interior<T, STATS, COLL, LAY>(h, s, src, dst);
+                if (h->g.ny > 2) e = launch_interior<T, STATS, COLL, LAY, false>(h, s, src, dst);
                 return e != cudaSuccess ? e : launch_wall_rows<T, STATS, COLL, LAY>(h, s, src, dst);
             } else {
                 // The odd step calls a separately compiled wall-row tile, which
@@ -313,17 +325,17 @@ cudaError_t launch_whole(lbm_handle *h, cudaStream_t s, const T *src, T *dst)
                     if (h->g.ny > 2)
                         return launch_ex(true, lbm::k_step_quad_aa_rows<STATS, COLL, LAY>, grid, block, 0, s, dst, h->g, h->p,
                                          h->tw, h->part);
-                return launch_ex(true, lbm::k_step_quad_aa<STATS, COLL, LAY, lbm::ROWS_ALL>, grid, block, 0, s, dst, h->g,
+                return launch_ex(true, lbm::k_step_quad_aa<STATS, COLL, LAY, lbm::ROWS_ALL, false>, grid, block, 0, s, dst, h->g,
                                  h->p, h->tw, h->part);
             }
         }
     }
     if constexpr (LAY == lbm::LAY_PULL)
         // read-only loads of the source lattice: no programmatic dependent launch
-        return launch_ex(!lbm::pull_nc<T>, lbm::k_step_pair<T, STATS, COLL, lbm::ROWS_ALL>, grid, block, 0, s, src, dst,
+        return launch_ex(!lbm::pull_nc<T>, lbm::k_step_pair<T, STATS, COLL, lbm::ROWS_ALL, false>, grid, block, 0, s, src, dst,
                          h->g, h->p, h->tw, h->part);
     else
-        return launch_ex(true, lbm::k_step_pair_aa<T, STATS, COLL, LAY, lbm::ROWS_ALL>, grid, block, 0, s, dst, h->g, h->p,
+        return launch_ex(true, lbm::k_step_pair_aa<T, STATS, COLL, LAY, lbm::ROWS_ALL, false>, grid, block, 0, s, dst, h->g, h->p,
                          h->tw, h->part);
 }
 
@@ -337,7 +349,9 @@ cudaError_t launch_lay(lbm_handle *h, cudaStream_t s, cudaStream_t s_wall, int s
     if (s_wall && !(LAY == lbm::LAY_AA_EVEN && whole_even_step(h))) {
         const cudaError_t e = launch_wall_rows<T, false, COLL, LAY>(h, s_wall, a, b);
         if (e != cudaSuccess) return e;
-        return launch_interior<T, false, COLL, LAY>(h, s, a, b);
+        if constexpr (LAY != lbm::LAY_AA_EVEN)   // even steps (phase 0) walk forwards
+            if (src && h->reverse) return launch_interior<T, false, COLL, LAY, true>(h, s, a, b);
+        return launch_interior<T, false, COLL, LAY, false>(h, s, a, b);
     }
     return stats ? launch_whole<T, true, COLL, LAY>(h, s, a, b) : launch_whole<T, false, COLL, LAY>(h, s, a, b);
 }

@@ -295,12 +295,13 @@ __device__ __forceinline__ long long push_offset(const Geom &g, int wall, int a,
     return (long long)slot * g.plane + ((long long)zt * g.ny + yt) * g.sx + xt;
 }
 
-// Row (y, z) of a step kernel's block.
+// Row (y, z) of a step kernel's block: the rows of the set in launch order, or
+// with REV its planes from the last to the first.
 enum { ROWS_ALL = 0, ROWS_INTERIOR = 1, ROWS_WALL = 2 };
-template <int ROWS>
+template <int ROWS, bool REV>
 __device__ __forceinline__ void row_of_block(const Geom &g, int &y, int &z)
 {
-    z = blockIdx.z;
+    z = REV ? g.nz - 1 - (int)blockIdx.z : (int)blockIdx.z;
     y = ROWS == ROWS_INTERIOR ? (int)blockIdx.y + 1
                               : (ROWS == ROWS_WALL ? (blockIdx.y == 0 ? 0 : g.ny - 1) : (int)blockIdx.y);
 }

@@ -33,6 +33,7 @@ struct lbm_handle {
     int tma_warps;               // warps per CTA of the row-pipelined kernel (4 or 8)
     int tma_stages;              // ring stages of the row-pipelined kernel
     int tma_smem;                // dynamic shared memory bytes of the row-pipelined kernel
+    bool reverse;                // steps from lattice or phase 1 walk the planes backwards
     int *err;                    // device flag set by a timed-out pipeline wait
     long long wait_limit;        // clock cycles a pipeline wait may take before it gives up
     cudaGraphExec_t chunk[2];    // kGraphSteps plain steps starting from cur = 0 / 1

@@ -401,7 +401,7 @@ __device__ __forceinline__ void cell_step(const T *src, T *dst, const Geom &g, c
 {
     const int x = blockIdx.x * blockDim.x + threadIdx.x;
     int y, z;
-    row_of_block<ROWS_ALL>(g, y, z);
+    row_of_block<ROWS_ALL, false>(g, y, z);
     const bool valid = x < g.nx;
     if (!STATS && !valid) return;
     const int xc = valid ? x : 0;

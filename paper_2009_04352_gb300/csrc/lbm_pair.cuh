@@ -663,14 +663,14 @@ __device__ __forceinline__ void pdl_begin()
 #define LBM_PAIR_MRT_MIN_BLOCKS 5   // the same for the MRT instantiations (96 registers)
 #endif
 
-template <typename T, bool STATS, int COLL, int ROWS>
+template <typename T, bool STATS, int COLL, int ROWS, bool REV>
 __global__ void __launch_bounds__(128, COLL == COLL_MRT ? LBM_PAIR_MRT_MIN_BLOCKS : LBM_PAIR_MIN_BLOCKS)
     k_step_pair(const T *__restrict__ src, T *__restrict__ dst, Geom g, Phys p, float *__restrict__ tw_out,
                 double *__restrict__ part)
 {
     pdl_begin();
     int y, z;
-    row_of_block<ROWS>(g, y, z);
+    row_of_block<ROWS, REV>(g, y, z);
     const long long blk = ((long long)y * g.nz + z) * gridDim.x + blockIdx.x;
     pair_tile<T, STATS, COLL, LAY_PULL, ROWS>(src, dst, g, p, tw_out, STATS ? part + blk * K_PART : nullptr, blockIdx.x,
                                               y, z);
@@ -688,20 +688,20 @@ __global__ void __launch_bounds__(256) k_step_pair_wall(const T *src, T *dst, Ge
 {
     pdl_begin();
     int y, z;
-    row_of_block<ROWS_WALL>(g, y, z);
+    row_of_block<ROWS_WALL, false>(g, y, z);
     const long long blk = ((long long)y * g.nz + z) * gridDim.x + blockIdx.x;
     pair_tile<T, STATS, COLL, LAY, ROWS_WALL>(src, dst, g, p, tw_out, STATS ? part + blk * K_PART : nullptr,
                                               blockIdx.x, y, z);
 }
 
 // The two-cell step on the single AA array (LAY_AA_EVEN or LAY_AA_ODD).
-template <typename T, bool STATS, int COLL, int LAY, int ROWS>
+template <typename T, bool STATS, int COLL, int LAY, int ROWS, bool REV>
 __global__ void __launch_bounds__(128, COLL == COLL_MRT ? LBM_PAIR_MRT_MIN_BLOCKS : LBM_PAIR_MIN_BLOCKS)
     k_step_pair_aa(T *f, Geom g, Phys p, float *__restrict__ tw_out, double *__restrict__ part)
 {
     pdl_begin();
     int y, z;
-    row_of_block<ROWS>(g, y, z);
+    row_of_block<ROWS, REV>(g, y, z);
     const long long blk = ((long long)y * g.nz + z) * gridDim.x + blockIdx.x;
     pair_tile<T, STATS, COLL, LAY, ROWS>(f, f, g, p, tw_out, STATS ? part + blk * K_PART : nullptr, blockIdx.x, y, z);
 }

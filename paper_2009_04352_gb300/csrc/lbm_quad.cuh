@@ -304,7 +304,7 @@ __device__ __forceinline__ void quad_tile(const __half *src, __half *dst, const 
 // (ROWS_INTERIOR, row blockIdx.y + 1) or 2 (ROWS_WALL, rows 0 and ny - 1).
 // The step runs as an interior launch and a wall-row launch, so that the wall
 // layer's code does not shape the register allocation of the interior rows.
-template <bool STATS, int COLL, int ROWS>
+template <bool STATS, int COLL, int ROWS, bool REV>
 __global__ void __launch_bounds__(128, COLL == COLL_MRT ? LBM_QUAD_MRT_MIN_BLOCKS
                                                          : (STATS ? LBM_QUAD_STATS_MIN_BLOCKS : LBM_QUAD_MIN_BLOCKS))
     k_step_quad(const __half *__restrict__ src,
@@ -314,7 +314,7 @@ __global__ void __launch_bounds__(128, COLL == COLL_MRT ? LBM_QUAD_MRT_MIN_BLOCK
 {
     pdl_begin();
     int y, z;
-    row_of_block<ROWS>(g, y, z);
+    row_of_block<ROWS, REV>(g, y, z);
     const long long blk = ((long long)y * g.nz + z) * gridDim.x + blockIdx.x;
     quad_tile<STATS, COLL, LAY_PULL, ROWS>(src, dst, g, p, tw_out, STATS ? part + blk * K_PART : nullptr,
                                            blockIdx.x, y, z);
@@ -342,7 +342,7 @@ __global__ void __launch_bounds__(128, COLL == COLL_MRT ? LBM_QUAD_MRT_MIN_BLOCK
 {
     pdl_begin();
     int y, z;
-    row_of_block<ROWS_ALL>(g, y, z);
+    row_of_block<ROWS_ALL, false>(g, y, z);
     const long long blk = ((long long)y * g.nz + z) * gridDim.x + blockIdx.x;
     double *pb = STATS ? part + blk * K_PART : nullptr;
     if (y == 0 || y == g.ny - 1)
@@ -354,7 +354,7 @@ __global__ void __launch_bounds__(128, COLL == COLL_MRT ? LBM_QUAD_MRT_MIN_BLOCK
 // The four-cell step on the single AA array (LAY_AA_EVEN or LAY_AA_ODD) over
 // the row set ROWS (grid.y ny, or ny - 2 for the interior rows, row
 // blockIdx.y + 1).
-template <bool STATS, int COLL, int LAY, int ROWS>
+template <bool STATS, int COLL, int LAY, int ROWS, bool REV>
 __global__ void __launch_bounds__(128, COLL == COLL_MRT ? LBM_QUAD_MRT_MIN_BLOCKS
                                                          : (STATS ? LBM_QUAD_STATS_MIN_BLOCKS : LBM_QUAD_AA_MIN_BLOCKS))
     k_step_quad_aa(__half *f, Geom g, Phys p,
@@ -363,7 +363,7 @@ __global__ void __launch_bounds__(128, COLL == COLL_MRT ? LBM_QUAD_MRT_MIN_BLOCK
 {
     pdl_begin();
     int y, z;
-    row_of_block<ROWS>(g, y, z);
+    row_of_block<ROWS, REV>(g, y, z);
     const long long blk = ((long long)y * g.nz + z) * gridDim.x + blockIdx.x;
     quad_tile<STATS, COLL, LAY, ROWS, ROWS == ROWS_INTERIOR>(f, f, g, p, tw_out, STATS ? part + blk * K_PART : nullptr, blockIdx.x, y, z);
 }
@@ -386,7 +386,7 @@ __global__ void __launch_bounds__(128, LBM_QUAD_AA_ROWS_MIN_BLOCKS)
 {
     pdl_begin();
     int y, z;
-    row_of_block<ROWS_ALL>(g, y, z);
+    row_of_block<ROWS_ALL, false>(g, y, z);
     const long long blk = ((long long)y * g.nz + z) * gridDim.x + blockIdx.x;
     double *pb = STATS ? part + blk * K_PART : nullptr;
     if (y == 0 || y == g.ny - 1)
