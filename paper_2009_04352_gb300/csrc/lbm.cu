@@ -8,6 +8,7 @@
 #include <algorithm>
 
 #include "lbm.h"
+#include "lbm_fields.cuh"
 #include "lbm_quad.cuh"
 #include "lbm_tma.cuh"
 
@@ -479,17 +480,70 @@ int ensure_part(lbm_handle *h, long long len)
     return LBM_OK;
 }
 
-int export_state(lbm_handle *h, float *rho, float *u, double *pops, double *part)
+// Populations (FP64, dense) or the per-block FP64 sums of k_export, one cell per
+// thread.
+int export_state(lbm_handle *h, double *pops, double *part)
 {
     const int bx = 128;
     const dim3 grid = grid_of(h, bx);
     const int map = lbm_state_map(h);
     if (h->precision == LBM_FP16_SHIFTED)
-        lbm::k_export<__half><<<grid, bx, 0, h->stream>>>((const __half *)lbm_state_ptr(h), h->g, h->p, map, rho, u,
-                                                          pops, part);
+        lbm::k_export<__half><<<grid, bx, 0, h->stream>>>((const __half *)lbm_state_ptr(h), h->g, h->p, map, pops, part);
     else
-        lbm::k_export<float><<<grid, bx, 0, h->stream>>>((const float *)lbm_state_ptr(h), h->g, h->p, map, rho, u,
-                                                         pops, part);
+        lbm::k_export<float><<<grid, bx, 0, h->stream>>>((const float *)lbm_state_ptr(h), h->g, h->p, map, pops, part);
+    CK_LAUNCH();
+    return LBM_OK;
+}
+
+// sum f - 1 and sum e f with FP64 additions per cell (any magnitude).
+int conservation_fp64(lbm_handle *h, double *out)
+{
+    const dim3 grid = grid_of(h, 128);
+    const long long nblk = (long long)grid.x * grid.y * grid.z;
+    double *d = nullptr;
+    if (cudaMallocAsync((void **)&d, (size_t)(nblk * 4 + 4) * sizeof(double), h->stream) != cudaSuccess)
+        return fail(LBM_ERR_OOM, "conservation buffer");
+    const int rc = export_state(h, nullptr, d);
+    if (rc != LBM_OK) return rc;
+    lbm::k_reduce_all<<<1, 256, 0, h->stream>>>(d, nblk, d + nblk * 4);
+    CK_LAUNCH();
+    CK(cudaMemcpyAsync(out, d + nblk * 4, 4 * sizeof(double), cudaMemcpyDeviceToHost, h->stream));
+    CK(cudaFreeAsync(d, h->stream));
+    CK(cudaStreamSynchronize(h->stream));
+    return LBM_OK;
+}
+
+template <typename T, int V, int LAY>
+void launch_moments(lbm_handle *h, float *rho, float *u)
+{
+    const int per_row = h->g.nx / V, bx = lbm::row_threads(per_row);
+    const bool wide = (((uintptr_t)rho | (uintptr_t)u) & (4 * V - 1)) == 0;
+    lbm::k_moments<T, V, LAY><<<dim3((per_row + bx - 1) / bx, h->g.ny, h->g.nz), bx, 0, h->stream>>>(
+        (const T *)lbm_state_ptr(h), h->g, h->p, rho, u, wide);
+}
+
+template <typename T, int V>
+void launch_moments_map(lbm_handle *h, float *rho, float *u)
+{
+    const int map = lbm_state_map(h);
+    if (map == lbm::MAP_AA0)
+        launch_moments<T, V, lbm::LAY_AA_EVEN>(h, rho, u);
+    else if (map == lbm::MAP_AA1)
+        launch_moments<T, V, lbm::LAY_AA_ODD>(h, rho, u);
+    else
+        launch_moments<T, V, lbm::LAY_PULL>(h, rho, u);
+}
+
+// Density and velocity into device arrays, with the widest gather the row
+// length allows (us a call, one cell a thread / here: see lbm_fields.cuh).
+int export_moments(lbm_handle *h, float *rho, float *u)
+{
+    const bool half = h->precision == LBM_FP16_SHIFTED;
+    switch (lbm::cells_wide(h)) {
+    case 1: half ? launch_moments_map<__half, 1>(h, rho, u) : launch_moments_map<float, 1>(h, rho, u); break;
+    case 2: half ? launch_moments_map<__half, 2>(h, rho, u) : launch_moments_map<float, 2>(h, rho, u); break;
+    default: launch_moments_map<__half, 4>(h, rho, u);
+    }
     CK_LAUNCH();
     return LBM_OK;
 }
@@ -752,7 +806,7 @@ int lbm_populations(lbm_handle *h, double *host_out)
     const size_t b = (size_t)lbm::Q * h->g.nx * h->g.ny * h->g.nz * sizeof(double);
     double *d = nullptr;
     if (cudaMallocAsync((void **)&d, b, h->stream) != cudaSuccess) return fail(LBM_ERR_OOM, "staging buffer");
-    int rc = export_state(h, nullptr, nullptr, d, nullptr);
+    int rc = export_state(h, d, nullptr);
     if (rc != LBM_OK) return rc;
     CK(cudaMemcpyAsync(host_out, d, b, cudaMemcpyDeviceToHost, h->stream));
     CK(cudaFreeAsync(d, h->stream));
@@ -876,12 +930,12 @@ int lbm_moments(lbm_handle *h, float *rho, float *u, int on_device)
     LbmRange range("lbm_moments");
     if (!h) return fail(LBM_ERR_ARG, "NULL handle");
     if (!rho && !u) return LBM_OK;
-    if (on_device) return export_state(h, rho, u, nullptr, nullptr);
+    if (on_device) return export_moments(h, rho, u);
     const long long n = (long long)h->g.nx * h->g.ny * h->g.nz;
     float *d = nullptr;
     if (cudaMallocAsync((void **)&d, (size_t)4 * n * sizeof(float), h->stream) != cudaSuccess)
         return fail(LBM_ERR_OOM, "staging buffer");
-    int rc = export_state(h, d, d + n, nullptr, nullptr);
+    int rc = export_moments(h, d, d + n);
     if (rc != LBM_OK) return rc;
     if (rho) CK(cudaMemcpyAsync(rho, d, (size_t)n * sizeof(float), cudaMemcpyDeviceToHost, h->stream));
     if (u) CK(cudaMemcpyAsync(u, d + n, (size_t)3 * n * sizeof(float), cudaMemcpyDeviceToHost, h->stream));
@@ -921,19 +975,23 @@ int lbm_conservation(lbm_handle *h, double *out)
 {
     LbmRange range("lbm_conservation");
     if (!h || !out) return fail(LBM_ERR_ARG, "NULL argument");
-    const dim3 grid = grid_of(h, 128);
-    const long long nblk = (long long)grid.x * grid.y * grid.z;
-    double *d = nullptr;
-    if (cudaMallocAsync((void **)&d, (size_t)(nblk * 4 + 4) * sizeof(double), h->stream) != cudaSuccess)
-        return fail(LBM_ERR_OOM, "conservation buffer");
-    int rc = export_state(h, nullptr, nullptr, nullptr, d);
-    if (rc != LBM_OK) return rc;
-    lbm::k_reduce_all<<<1, 256, 0, h->stream>>>(d, nblk, d + nblk * 4);
+    // the partials lie in the handle's buffer of the sampled steps' partials,
+    // which holds K_PART > 4 sums for every row tile
+    const int blocks = lbm::plane_sum_blocks(h, 1 << 30);
+    const long long nblk = (long long)blocks * h->g.ny;
+    lbm::plane_sums<false>(h, blocks, h->part);
     CK_LAUNCH();
-    CK(cudaMemcpyAsync(out, d + nblk * 4, 4 * sizeof(double), cudaMemcpyDeviceToHost, h->stream));
-    CK(cudaFreeAsync(d, h->stream));
-    rc = check_err(h);
+    lbm::k_reduce_all<<<1, 256, 0, h->stream>>>(h->part, nblk, h->part + nblk * 4);
+    CK_LAUNCH();
+    CK(cudaMemcpyAsync(out, h->part + nblk * 4, 4 * sizeof(double), cudaMemcpyDeviceToHost, h->stream));
+    int rc = check_err(h);
     if (rc != LBM_OK) return rc;
+    if (!(isfinite(out[0]) && isfinite(out[1]) && isfinite(out[2]) && isfinite(out[3]))) {
+        // NaN or infinite populations, or finite ones so large that an FP32 sum
+        // overflowed: the FP64 sums per cell tell which
+        rc = conservation_fp64(h, out);
+        if (rc != LBM_OK) return rc;
+    }
     // the partials are deviations from the rest state: add sum w = 1 per cell
     out[0] += (double)h->g.nx * h->g.ny * h->g.nz;
     for (int k = 0; k < 4; ++k)

@@ -519,11 +519,9 @@ static __global__ void k_reduce_planes(const double *__restrict__ part, long lon
 }
 
 // Exports of the current populations f(t) (gathered exactly as the step does):
-// moments (FP32), unshifted populations (FP64) and FP64 block partials of
-// (sum f - 1, sum e f) for the conservation check.
+// unshifted populations (FP64) and FP64 block partials of (sum f - 1, sum e f).
 template <typename T>
 __global__ void __launch_bounds__(256) k_export(const T *__restrict__ src, Geom g, Phys p, int map,
-                                                float *__restrict__ rho_out, float *__restrict__ u_out,
                                                 double *__restrict__ pop_out, double *__restrict__ part)
 {
     const int x = blockIdx.x * blockDim.x + threadIdx.x;
@@ -534,20 +532,9 @@ __global__ void __launch_bounds__(256) k_export(const T *__restrict__ src, Geom 
     gather_any<T>(src, g, p.wall, map, xc, y, z, f);
     const long long n = (long long)g.nx * g.ny * g.nz;
     const long long cell = ((long long)z * g.ny + y) * g.nx + x;
-    if (valid) {
-        if (rho_out || u_out) {
-            const CellState c = velocity(moments_of(f), p);
-            if (rho_out) rho_out[cell] = c.rho;
-            if (u_out) {
-                u_out[cell] = c.ux;
-                u_out[n + cell] = c.uy;
-                u_out[2 * n + cell] = c.uz;
-            }
-        }
-        if (pop_out) {
+    if (valid && pop_out) {
 #pragma unroll
-            for (int a = 0; a < Q; ++a) pop_out[a * n + cell] = (double)f[a] + w_of(a);
-        }
+        for (int a = 0; a < Q; ++a) pop_out[a * n + cell] = (double)f[a] + w_of(a);
     }
     if (part) {
         double v[4] = {0.0, 0.0, 0.0, 0.0};
