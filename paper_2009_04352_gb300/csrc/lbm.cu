@@ -9,6 +9,7 @@
 
 #include "lbm.h"
 #include "lbm_fields.cuh"
+#include "lbm_odd.cuh"
 #include "lbm_quad.cuh"
 #include "lbm_tma.cuh"
 
@@ -245,9 +246,15 @@ constexpr long long kSplitFp32Min = 1LL << 18, kSplitFp32Max = 1LL << 25;
 // (256x64x128: 27.7 against 27.1, 128x48x96: 11.1 against 10.0).
 constexpr long long kWholeEvenCells = 1LL << 23;
 
+// Whether plain steps of the one-cell form run two cells a thread (lbm_odd.cuh).
+bool odd_step(const lbm_handle *h)
+{
+    return h->kernel == LBM_KERNEL_CELL && h->g.nx % 2 == 1 && h->p.wall != lbm::WALL_NODE;
+}
+
 bool split_step(const lbm_handle *h)
 {
-    if ((h->kernel != LBM_KERNEL_PAIR && h->kernel != LBM_KERNEL_QUAD) || h->g.ny < 3) return false;
+    if (h->kernel == LBM_KERNEL_TMA || (h->kernel == LBM_KERNEL_CELL && !odd_step(h)) || h->g.ny < 3) return false;
     const long long cells = (long long)h->g.nx * h->g.ny * h->g.nz;
     if (h->precision == LBM_FP32 && h->layout == LBM_PULL2) return cells >= kSplitFp32Min && cells < kSplitFp32Max;
     return true;
@@ -258,10 +265,22 @@ bool whole_even_step(const lbm_handle *h)
     return h->kernel == LBM_KERNEL_QUAD && (long long)h->g.nx * h->g.ny * h->g.nz >= kWholeEvenCells;
 }
 
+// A plain step of odd_step over a row set.
+template <typename T, int COLL, int LAY, int ROWS, bool REV>
+cudaError_t launch_odd(lbm_handle *h, cudaStream_t s, const T *src, T *dst)
+{
+    const int pairs = (h->g.nx + 1) / 2, bx = lbm::row_threads(pairs);
+    const int rows = ROWS == lbm::ROWS_INTERIOR ? h->g.ny - 2 : (ROWS == lbm::ROWS_WALL ? 2 : h->g.ny);
+    return launch_ex(LAY != lbm::LAY_PULL || !lbm::pull_nc<T>, lbm::k_step_odd<T, COLL, LAY, ROWS, REV>,
+                     dim3((pairs + bx - 1) / bx, rows, h->g.nz), dim3(bx), 0, s, src, dst, h->g, h->p, h->tw);
+}
+
 // The two wall rows of a step in a launch of their own, with the two-cell tile.
 template <typename T, bool STATS, int COLL, int LAY>
 cudaError_t launch_wall_rows(lbm_handle *h, cudaStream_t s, const T *src, T *dst)
 {
+    if constexpr (!STATS)
+        if (h->kernel == LBM_KERNEL_CELL) return launch_odd<T, COLL, LAY, lbm::ROWS_WALL, false>(h, s, src, dst);
     const dim3 all = step_grid(h), grid(all.x, 2, all.z);
     const dim3 block(h->kernel == LBM_KERNEL_QUAD ? 2 * h->bx : h->bx);
     return launch_ex(LAY != lbm::LAY_PULL || !lbm::pull_nc<T>, lbm::k_step_pair_wall<T, STATS, COLL, LAY>, grid, block, 0, s, src,
@@ -272,6 +291,8 @@ cudaError_t launch_wall_rows(lbm_handle *h, cudaStream_t s, const T *src, T *dst
 template <typename T, bool STATS, int COLL, int LAY, bool REV>
 cudaError_t launch_interior(lbm_handle *h, cudaStream_t s, const T *src, T *dst)
 {
+    if constexpr (!STATS)
+        if (h->kernel == LBM_KERNEL_CELL) return launch_odd<T, COLL, LAY, lbm::ROWS_INTERIOR, REV>(h, s, src, dst);
     const dim3 all = step_grid(h), grid(all.x, h->g.ny - 2, all.z), block(h->bx);
     if constexpr (sizeof(T) == 2) {
         if (h->kernel == LBM_KERNEL_QUAD) {
@@ -298,6 +319,8 @@ cudaError_t launch_whole(lbm_handle *h, cudaStream_t s, const T *src, T *dst)
 {
     const dim3 grid = step_grid(h), block(h->bx);
     if (h->kernel == LBM_KERNEL_CELL) {
+        if constexpr (!STATS)
+            if (odd_step(h)) return launch_odd<T, COLL, LAY, lbm::ROWS_ALL, false>(h, s, src, dst);
         if constexpr (LAY == lbm::LAY_PULL)
             return launch_ex(false, lbm::k_step<T, STATS, COLL>, grid, block, 0, s, src, dst, h->g, h->p, h->tw, h->part);
         else
