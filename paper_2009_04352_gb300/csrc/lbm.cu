@@ -59,6 +59,15 @@ dim3 step_grid(const lbm_handle *h)
 
 int configure_rows(lbm_handle *h);
 
+void drop_graphs(lbm_handle *h)
+{
+    for (int i = 0; i < 2; ++i) {
+        if (h->chunk[i]) cudaGraphExecDestroy(h->chunk[i]);
+        if (h->period[i]) cudaGraphExecDestroy(h->period[i]);
+        h->chunk[i] = h->period[i] = nullptr;
+    }
+}
+
 int select_kernel(lbm_handle *h, int kernel)
 {
     const bool even = (h->g.nx % 2) == 0;
@@ -99,11 +108,7 @@ int select_kernel(lbm_handle *h, int kernel)
         if (rc != LBM_OK) return rc;
     }
     // captured graphs hold the old launch configuration
-    for (int i = 0; i < 2; ++i)
-        if (h->chunk[i]) {
-            cudaGraphExecDestroy(h->chunk[i]);
-            h->chunk[i] = nullptr;
-        }
+    drop_graphs(h);
     return LBM_OK;
 }
 
@@ -431,15 +436,17 @@ int launch_step(lbm_handle *h, cudaStream_t s, int src, bool stats, cudaStream_t
                                            : launch_step_c<lbm::COLL_BGK>(h, s, src, stats, s_wall);
 }
 
-int build_chunk(lbm_handle *h, int start)
+// Graph of `steps` steps from lattice (or phase) start, the first one sampled
+// when `sample`.
+int build_graph(lbm_handle *h, int start, int steps, bool sample, cudaGraphExec_t *out)
 {
     cudaGraph_t graph = nullptr;
     CK(cudaStreamBeginCapture(h->cap, cudaStreamCaptureModeThreadLocal));
     int rc = LBM_OK;
     const bool fork = split_step(h);
     cudaError_t ce = cudaSuccess;
-    for (int i = 0; i < kGraphSteps && rc == LBM_OK && ce == cudaSuccess; ++i) {
-        if (fork) {
+    for (int i = 0; i < steps && rc == LBM_OK && ce == cudaSuccess; ++i) {
+        if (fork && !(sample && i == 0)) {
             // the step's two launches depend on the whole previous step and
             // the next step on both of them
             ce = cudaEventRecord(h->fork, h->cap);
@@ -448,7 +455,7 @@ int build_chunk(lbm_handle *h, int start)
             if (ce == cudaSuccess && rc == LBM_OK) ce = cudaEventRecord(h->join, h->cap_wall);
             if (ce == cudaSuccess && rc == LBM_OK) ce = cudaStreamWaitEvent(h->cap, h->join, 0);
         } else {
-            rc = launch_step(h, h->cap, start ^ (i & 1), false);
+            rc = launch_step(h, h->cap, start ^ (i & 1), sample && i == 0);
         }
     }
     cudaError_t e = cudaStreamEndCapture(h->cap, &graph);
@@ -458,25 +465,41 @@ int build_chunk(lbm_handle *h, int start)
         return rc;
     }
     if (e != cudaSuccess) return fail(LBM_ERR_CUDA, "graph capture: %s", cudaGetErrorString(e));
-    e = cudaGraphInstantiate(&h->chunk[start], graph, 0);
+    e = cudaGraphInstantiate(out, graph, 0);
     cudaGraphDestroy(graph);
     if (e != cudaSuccess) return fail(LBM_ERR_CUDA, "graph instantiate: %s", cudaGetErrorString(e));
     // move the graph's device-side set-up off its first launch
-    e = cudaGraphUpload(h->chunk[start], h->stream);
+    e = cudaGraphUpload(*out, h->stream);
     if (e != cudaSuccess) return fail(LBM_ERR_CUDA, "graph upload: %s", cudaGetErrorString(e));
     return LBM_OK;
 }
 
 // Both chunk graphs (start phase 0 and 1), built together on the first step
 // call after any change that invalidated them, whatever the step count, so that
-// no capture or instantiation falls inside a later, longer run of steps.
+// no capture or instantiation falls inside a later, longer run of steps. With
+// sampling, also the graphs of a sampled step and the plain steps after it that
+// do not fill a chunk (an interval of 10 would otherwise never reach one: of
+// 252x80x126 MRT every plain step then ran as a single launch, 70 us against 66).
 int ensure_chunks(lbm_handle *h)
 {
     for (int start = 0; start < 2; ++start)
         if (!h->chunk[start]) {
-            const int rc = build_chunk(h, start);
+            const int rc = build_graph(h, start, kGraphSteps, false, &h->chunk[start]);
             if (rc != LBM_OK) return rc;
         }
+    const int len = h->stats_every > 0 ? 1 + (h->stats_every - 1) % kGraphSteps : 0;
+    if (len < 2) return LBM_OK;
+    for (int start = 0; start < 2; ++start) {
+        if (h->period[start] && h->period_len == len) continue;
+        if (h->period[start]) {
+            CK(cudaStreamSynchronize(h->stream));   // it may be in flight
+            cudaGraphExecDestroy(h->period[start]);
+            h->period[start] = nullptr;
+        }
+        const int rc = build_graph(h, start, len, true, &h->period[start]);
+        if (rc != LBM_OK) return rc;
+        if (start == 1) h->period_len = len;
+    }
     return LBM_OK;
 }
 
@@ -495,11 +518,7 @@ int ensure_part(lbm_handle *h, long long len)
     }
     h->part_len = len;
     // the partial buffer is captured by address in the chunk graphs
-    for (int i = 0; i < 2; ++i)
-        if (h->chunk[i]) {
-            cudaGraphExecDestroy(h->chunk[i]);
-            h->chunk[i] = nullptr;
-        }
+    drop_graphs(h);
     return LBM_OK;
 }
 
@@ -737,10 +756,9 @@ void lbm_free_handle(lbm_handle *h)
 {
     if (!h) return;
     if (h->stream || h->f[0]) cudaStreamSynchronize(h->stream);
-    for (int i = 0; i < 2; ++i) {
-        if (h->chunk[i]) cudaGraphExecDestroy(h->chunk[i]);
+    drop_graphs(h);
+    for (int i = 0; i < 2; ++i)
         if (h->f[i] && !h->borrowed) cudaFree(h->f[i]);
-    }
     if (h->part) cudaFree(h->part);
     if (h->tw) cudaFree(h->tw);
     if (h->acc) cudaFree(h->acc);
@@ -854,6 +872,14 @@ int lbm_step(lbm_handle *h, int n)
     }
     while (n > 0) {
         const bool sample = h->stats_every > 0 && (h->step % h->stats_every) == 0;
+        if (sample && h->stats_every % kGraphSteps != 1 && n >= h->period_len) {
+            CK(cudaGraphLaunch(h->period[h->cur], h->stream));
+            h->nsamples += 1;
+            h->cur ^= h->period_len & 1;
+            h->step += h->period_len;
+            n -= h->period_len;
+            continue;
+        }
         if (sample) {
             int rc = launch_step(h, h->stream, h->cur, true);
             if (rc != LBM_OK) return rc;
@@ -1028,11 +1054,7 @@ int lbm_set_wait_limit(lbm_handle *h, long long cycles)
     CK(cudaStreamSynchronize(h->stream));
     h->wait_limit = cycles > 0 ? cycles : lbm::WAIT_CYCLES;
     // captured graphs hold the old limit
-    for (int i = 0; i < 2; ++i)
-        if (h->chunk[i]) {
-            cudaGraphExecDestroy(h->chunk[i]);
-            h->chunk[i] = nullptr;
-        }
+    drop_graphs(h);
     return LBM_OK;
 }
 

@@ -37,6 +37,8 @@ struct lbm_handle {
     int *err;                    // device flag set by a timed-out pipeline wait
     long long wait_limit;        // clock cycles a pipeline wait may take before it gives up
     cudaGraphExec_t chunk[2];    // kGraphSteps plain steps starting from cur = 0 / 1
+    cudaGraphExec_t period[2];   // a sampled step and the period_len - 1 plain ones after it, from cur = 0 / 1
+    int period_len;
     bool member;                 // member view of a batch (stepped by the batch)
     bool borrowed;               // population arrays owned by the caller or a batch, not freed here
     double nu_wall;              // viscosity of the wall law and of the van Driest y+
