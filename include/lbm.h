@@ -217,14 +217,14 @@ int lbm_set_stats_every(lbm_handle *h, int every);
 
 /* Advance n >= 0 time steps (Eq. 1 with the wall treatment of Eqs. 14-17).
  * Asynchronous on the handle's stream; steps without sampling are replayed
- * from CUDA graphs of 16 steps. The first call with n > 0 after lbm_create,
+ * from CUDA graphs of a few sizes (up to 16 steps). The first call with n > 0 after lbm_create,
  * lbm_set_kernel, lbm_set_les or lbm_set_wait_limit captures, instantiates and
- * uploads both of those graphs (one per start phase), whatever n is, so a
+ * uploads all of those graphs, whatever n is, so a
  * short warm-up call leaves nothing to build inside a later timed run; make
  * that first call outside any stream capture of the caller's own. With
- * sampling every k steps, k not 1 more than a multiple of 16, a sampled step and
- * the (k - 1) % 16 plain steps after it are a graph too, built likewise on the
- * first call after lbm_set_stats_every changed k. */
+ * sampling every k steps, a sampled step and the plain steps after it that do
+ * not fill a graph are a graph too, built likewise on the first call after
+ * lbm_set_stats_every changed k. */
 int lbm_step(lbm_handle *h, int n);
 
 /* Number of steps taken since the last (re)initialisation. */

@@ -35,7 +35,11 @@
 
 namespace {
 
-constexpr int kBatchGraphSteps = 16;
+// Steps of the graphs that plain runs are made of: chunks of 16 from lattice 0,
+// then quarters of 4 and single steps from either lattice (26 captured steps in
+// all, where a chunk for each lattice was 32). Outside a graph the members run
+// one after the other on one stream.
+constexpr int kBatchGraphSteps = 16, kBatchQuarterSteps = 4;
 constexpr int kMaxStreams = 32;   // capture streams of the member-grid form
 
 struct BatchInst {
@@ -155,7 +159,7 @@ struct lbm_batch {
     int cur;
     long long step;
     int stats_every;
-    cudaGraphExec_t chunk[2];
+    cudaGraphExec_t chunk, quarter[2], one[2];
 };
 
 namespace {
@@ -164,10 +168,10 @@ size_t elem_bytes(int precision) { return precision == LBM_FP16_SHIFTED ? 2 : 4;
 
 void drop_graphs(lbm_batch *b)
 {
-    for (int i = 0; i < 2; ++i)
-        if (b->chunk[i]) {
-            cudaGraphExecDestroy(b->chunk[i]);
-            b->chunk[i] = nullptr;
+    for (cudaGraphExec_t *g : {&b->chunk, &b->quarter[0], &b->quarter[1], &b->one[0], &b->one[1]})
+        if (*g) {
+            cudaGraphExecDestroy(*g);
+            *g = nullptr;
         }
 }
 
@@ -297,7 +301,8 @@ int launch(lbm_batch *b, cudaStream_t s, int cur, bool stats)
     return LBM_OK;
 }
 
-int build_chunk(lbm_batch *b, int start)
+// Graph of `steps` plain steps of all members from lattice start.
+int build_graph(lbm_batch *b, int start, int steps, cudaGraphExec_t *out)
 {
     cudaGraph_t graph = nullptr;
     BK(cudaStreamBeginCapture(b->cap, cudaStreamCaptureModeThreadLocal));
@@ -311,7 +316,7 @@ int build_chunk(lbm_batch *b, int start)
         // they fit (step by step over the stream's members, 64 channels of 4096
         // to 262144 cells took 5965 us for 32 steps, this way 5137)
         for (int m = 0; m < b->n && rc == LBM_OK; ++m)
-            for (int i = 0; i < kBatchGraphSteps && rc == LBM_OK; ++i)
+            for (int i = 0; i < steps && rc == LBM_OK; ++i)
                 rc = lbm_launch_step(b->members[m], b->side[b->lane[m]], start ^ (i & 1), false);
         for (int k = 0; k < b->nstreams && ce == cudaSuccess; ++k) {
             ce = cudaEventRecord(b->join[k], b->side[k]);
@@ -319,7 +324,7 @@ int build_chunk(lbm_batch *b, int start)
         }
         if (ce != cudaSuccess && rc == LBM_OK) rc = fail_cuda(ce, "graph join");
     } else {
-        for (int i = 0; i < kBatchGraphSteps && rc == LBM_OK; ++i) rc = launch(b, b->cap, start ^ (i & 1), false);
+        for (int i = 0; i < steps && rc == LBM_OK; ++i) rc = launch(b, b->cap, start ^ (i & 1), false);
     }
     cudaError_t e = cudaStreamEndCapture(b->cap, &graph);
     if (rc != LBM_OK) {
@@ -327,24 +332,25 @@ int build_chunk(lbm_batch *b, int start)
         return rc;
     }
     if (e != cudaSuccess) return fail_cuda(e, "graph capture");
-    e = cudaGraphInstantiate(&b->chunk[start], graph, 0);
+    e = cudaGraphInstantiate(out, graph, 0);
     cudaGraphDestroy(graph);
     if (e != cudaSuccess) return fail_cuda(e, "graph instantiate");
-    e = cudaGraphUpload(b->chunk[start], b->stream);
+    e = cudaGraphUpload(*out, b->stream);
     if (e != cudaSuccess) return fail_cuda(e, "graph upload");
     return LBM_OK;
 }
 
-// Both chunk graphs, built on the first step call after a reconfiguration
-// (whatever its step count), so that no capture lands inside a later run.
+// All graphs, built on the first step call after a reconfiguration (whatever
+// its step count), so that no capture lands inside a later run.
 int ensure_chunks(lbm_batch *b)
 {
-    for (int start = 0; start < 2; ++start)
-        if (!b->chunk[start]) {
-            const int rc = build_chunk(b, start);
-            if (rc != LBM_OK) return rc;
-        }
-    return LBM_OK;
+    int rc = LBM_OK;
+    if (!b->chunk) rc = build_graph(b, 0, kBatchGraphSteps, &b->chunk);
+    for (int start = 0; start < 2 && rc == LBM_OK; ++start) {
+        if (!b->quarter[start]) rc = build_graph(b, start, kBatchQuarterSteps, &b->quarter[start]);
+        if (rc == LBM_OK && !b->one[start]) rc = build_graph(b, start, 1, &b->one[start]);
+    }
+    return rc;
 }
 
 void sync_members(lbm_batch *b)
@@ -373,7 +379,7 @@ int lbm_batch_create(int n, const lbm_member *members, int precision, void *cuda
     b->n = n;
     b->precision = precision;
     b->stream = (cudaStream_t)cuda_stream;
-    b->chunk[0] = b->chunk[1] = nullptr;
+    b->chunk = b->quarter[0] = b->quarter[1] = b->one[0] = b->one[1] = nullptr;
     b->pool = nullptr;
     b->d_inst = nullptr;
     b->cap = nullptr;
@@ -486,19 +492,22 @@ int lbm_batch_step(lbm_batch *b, int n)
         }
         long long run = n;
         if (b->stats_every > 0) run = std::min<long long>(run, b->stats_every - (b->step % b->stats_every));
-        while (run >= kBatchGraphSteps) {
-            BK(cudaGraphLaunch(b->chunk[b->cur], b->stream));
-            b->step += kBatchGraphSteps;
-            run -= kBatchGraphSteps;
-            n -= kBatchGraphSteps;
-        }
         while (run > 0) {
-            const int rc = launch(b, b->stream, b->cur, false);
-            if (rc != LBM_OK) return rc;
-            b->cur ^= 1;
-            b->step += 1;
-            run -= 1;
-            n -= 1;
+            int done;
+            if (b->cur == 0 && run >= kBatchGraphSteps) {
+                done = kBatchGraphSteps;
+                BK(cudaGraphLaunch(b->chunk, b->stream));
+            } else if (run >= kBatchQuarterSteps && run <= kBatchGraphSteps) {
+                done = kBatchQuarterSteps;
+                BK(cudaGraphLaunch(b->quarter[b->cur], b->stream));
+            } else {
+                done = 1;
+                BK(cudaGraphLaunch(b->one[b->cur], b->stream));
+                b->cur ^= 1;
+            }
+            b->step += done;
+            run -= done;
+            n -= done;
         }
     }
     sync_members(b);
