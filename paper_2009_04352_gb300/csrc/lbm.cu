@@ -88,7 +88,10 @@ int select_kernel(lbm_handle *h, int kernel)
     if (kernel < LBM_KERNEL_CELL || kernel > LBM_KERNEL_QUAD) return fail(LBM_ERR_ARG, "unknown kernel");
     h->kernel = kernel;
     const int per_row = h->g.nx / cells_per_thread(kernel);
-    h->bx = per_row >= 128 ? 128 : (per_row > 32 ? 64 : 32);   // <= the kernels' launch bound of 128
+    h->bx = row_threads(per_row);
+    // four-cell rows of just under four warps: two CTAs of two (448 cells: 43.3 us
+    // against 43.9)
+    if (kernel == LBM_KERNEL_QUAD && h->bx == 128 && per_row < 128) h->bx = 64;
     // Steps from lattice (or phase) 1 walk the planes backwards, so that each
     // step begins with the planes the step before wrote last, which L2 still
     // holds. Measured (us a step, forwards only / alternating): FP32 256x64x128
@@ -272,7 +275,7 @@ bool whole_even_step(const lbm_handle *h)
 template <typename T, int COLL, int LAY, int ROWS, bool REV>
 cudaError_t launch_odd(lbm_handle *h, cudaStream_t s, const T *src, T *dst)
 {
-    const int pairs = (h->g.nx + 1) / 2, bx = lbm::row_threads(pairs);
+    const int pairs = (h->g.nx + 1) / 2, bx = row_threads(pairs);
     const int rows = ROWS == lbm::ROWS_INTERIOR ? h->g.ny - 2 : (ROWS == lbm::ROWS_WALL ? 2 : h->g.ny);
     return launch_ex(LAY != lbm::LAY_PULL || !lbm::pull_nc<T>, lbm::k_step_odd<T, COLL, LAY, ROWS, REV>,
                      dim3((pairs + bx - 1) / bx, rows, h->g.nz), dim3(bx), 0, s, src, dst, h->g, h->p, h->tw);
@@ -570,7 +573,7 @@ int conservation_fp64(lbm_handle *h, double *out)
 template <typename T, int V, int LAY>
 void launch_moments(lbm_handle *h, float *rho, float *u)
 {
-    const int per_row = h->g.nx / V, bx = lbm::row_threads(per_row);
+    const int per_row = h->g.nx / V, bx = row_threads(per_row);
     const bool wide = (((uintptr_t)rho | (uintptr_t)u) & (4 * V - 1)) == 0;
     lbm::k_moments<T, V, LAY><<<dim3((per_row + bx - 1) / bx, h->g.ny, h->g.nz), bx, 0, h->stream>>>(
         (const T *)lbm_state_ptr(h), h->g, h->p, rho, u, wide);

@@ -6,7 +6,7 @@
 // of k_export with FP64 sums did not: FP64 runs at 1/64 of the FP32 rate here, and
 // FP16 storage was read 2 bytes at a time. us a call at 512x128x256, before / now
 // (floor, the reads and writes at the copy rate): conservation FP32 3980 / 388 (188),
-// FP16 3967 / 266 (94); plane profile FP32 739 / 353, AA 721 / 218 (188), FP16 736 /
+// FP16 3967 / 266 (94); plane profile FP32 739 / 306, AA 721 / 218 (188), FP16 736 /
 // 214 (94); moments FP32 234 / 220 (228), FP16 206 / 158, AA 181 / 133 (134). Here a thread gathers V cells of a row with the wide loads of the
 // step kernels (gather_pair, gather_quad), and the sums run in compensated FP32:
 // every addition is an error-free transformation (Knuth's two-sum; products with
@@ -240,8 +240,13 @@ __device__ __forceinline__ void profile_add_fp64(double (&v)[16], float rho, flo
 //            direction, combined in FP64
 // to out[(y gridDim.x + blockIdx.x) columns]. The order of the additions depends
 // on the grid only, so every layout and storage map gives the same bits.
+// CTAs per SM the register budget must allow (us at 512x128x256, 3 / 4 / 5): FP32
+// profile 342 / 353 / 306, FP16 profile 222 / 214 / 235, conservation FP32 462 / 386 /
+// 415, FP16 262 / 265 / 364.
+template <typename T, bool PROFILE> constexpr int SUM_BLOCKS = PROFILE && sizeof(T) == 4 ? 5 : 4;
+
 template <typename T, int V, int LAY, bool PROFILE>
-__global__ void __launch_bounds__(128, 4) k_plane_sums(const T *__restrict__ src, Geom g, Phys p, int nxb,
+__global__ void __launch_bounds__(128, SUM_BLOCKS<T, PROFILE>) k_plane_sums(const T *__restrict__ src, Geom g, Phys p, int nxb,
                                                        double *__restrict__ out)
 {
     constexpr int NP = (V + 1) / 2, NS = PROFILE ? K_STATS : Q, NOUT = PROFILE ? K_STATS : 4;
@@ -322,12 +327,11 @@ __global__ void __launch_bounds__(128, 4) k_plane_sums(const T *__restrict__ src
     if (threadIdx.x < NOUT) out[((long long)y * gridDim.x + blockIdx.x) * NOUT + threadIdx.x] = r;
 }
 
-// Cells a thread gathers at once on rows of nx cells, and the CTA's threads.
+// Cells a thread gathers at once on rows of nx cells.
 inline int cells_wide(const lbm_handle *h)
 {
     return h->g.nx % 2 ? 1 : (h->precision == LBM_FP16_SHIFTED && h->g.nx % 4 == 0 ? 4 : 2);
 }
-inline int row_threads(int per_row) { return per_row > 64 ? 128 : (per_row > 32 ? 64 : 32); }
 
 // CTAs of k_plane_sums for each plane: about four rounds of the four CTAs an SM
 // holds of the 152 of this GPU over all planes, at most one for each row tile and

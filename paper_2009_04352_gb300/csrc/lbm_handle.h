@@ -45,6 +45,18 @@ struct lbm_handle {
     double nu_wall;              // viscosity of the wall law and of the van Driest y+
 };
 
+// Threads of the CTAs that share a row of per_row threads' work: whole warps, at
+// most 128 (the kernels' launch bound), split evenly. A warp past the row end
+// costs a warp's issue slots: with CTAs of 32, 64 or 128 threads rows of 130 cells
+// ran six warps for three (FP32 103.2 us a step of 3M cells against 90.8, FP16 82.7
+// / 64.1), 320 cells eight for five (81.0 / 71.5, 57.6 / 46.6), 192 cells four for
+// three (74.3 / 68.7).
+inline int row_threads(int per_row)
+{
+    const int warps = (per_row + 31) / 32, tiles = (warps + 3) / 4;
+    return 32 * ((warps + tiles - 1) / tiles);
+}
+
 // The array holding the current state and the map under which f(t) is stored.
 inline void *lbm_state_ptr(const lbm_handle *h) { return h->layout == LBM_AA ? h->f[0] : h->f[h->cur]; }
 inline int lbm_state_map(const lbm_handle *h)

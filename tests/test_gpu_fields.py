@@ -87,3 +87,25 @@ def test_finite_sums_beyond_fp32_stay_finite():
         ch.conservation()
     assert ei.value.code == lbm.LBM_ERR_DIVERGED
     ch.close()
+
+
+@pytest.mark.parametrize("layout", [lbm.PULL2, lbm.AA])
+@pytest.mark.parametrize("precision", [lbm.FP32, lbm.FP16_SHIFTED])
+@pytest.mark.parametrize("nx", [66, 130, 192, 258, 322, 386, 452, 520, 151, 301])
+def test_sampled_sums_match_the_profile(nx, precision, layout):
+    """Rows of every number of warps a CTA takes (one to four) and several CTAs a
+    row: the fused sums of a sampled step against the profile of the state it
+    starts from (FP32 warp sums: a few 1e-7 of the column)."""
+    case = workload.derive_channel("rows", nx, 9, 7, 640.0)
+    ch = lbm.Channel.from_case(case, precision=precision, layout=layout)
+    ch.init_channel(workload.u_mean_profile(case), workload.noise_amplitude(case), 9)
+    prof = torch.empty((9, lbm.K_STATS), dtype=torch.float64, device="cuda")
+    for _ in range(2):
+        lbm.lbm_plane_profile_noalloc(ch.handle, prof.data_ptr())
+        ch.set_stats_every(1)
+        ch.step(1)
+        st, _, n = ch.plane_stats(reset=True)
+        assert n == 1
+        want = prof.cpu().numpy()
+        assert np.all(np.abs(st - want) <= 1e-6 * np.max(np.abs(want), axis=0))
+    ch.close()
