@@ -245,25 +245,29 @@ int configure_rows(lbm_handle *h)
 // 30.2 / 27.7, 64x32x32 8.6 / 5.4. The two-lattice FP32 step, bound by DRAM alone,
 // gains nothing at 512x128x256 (375.5 / 376.6) and loses 0.9% at 1024x256x512 (2961
 // / 2987), and at 64x32x32 it gains less than the larger graph costs to build, so
-// it is split between 2^18 and 2^25 cells.
-constexpr long long kSplitFp32Min = 1LL << 18, kSplitFp32Max = 1LL << 25;
+// it is split between 2^18 and 2^25 cells; FP32 AA from 2^16 (16x8x8: 20 steps 105
+// us whole, 113 split).
+constexpr long long kSplitFp32Min = 1LL << 18, kSplitFp32Max = 1LL << 25, kSplitFp32AaMin = 1LL << 16;
 // The even AA step of the four-cell kernel is better in one launch on large
 // grids (512x128x256 step pair: 208.1 against 214.1 us a step), on small ones not
 // (256x64x128: 27.7 against 27.1, 128x48x96: 11.1 against 10.0).
 constexpr long long kWholeEvenCells = 1LL << 23;
 
 // Whether plain steps of the one-cell form run two cells a thread (lbm_odd.cuh).
+// Below 2^17 cells the one-cell kernel's twice as many threads hide latency
+// better (99x20x28 FP32 6.3 us a step against 8.3; 125x20x131 13.5 against 11.4).
 bool odd_step(const lbm_handle *h)
 {
-    return h->kernel == LBM_KERNEL_CELL && h->g.nx % 2 == 1 && h->p.wall != lbm::WALL_NODE;
+    return h->kernel == LBM_KERNEL_CELL && h->g.nx % 2 == 1 && h->p.wall != lbm::WALL_NODE &&
+           (long long)h->g.nx * h->g.ny * h->g.nz >= 1LL << 17;
 }
 
 bool split_step(const lbm_handle *h)
 {
     if (h->kernel == LBM_KERNEL_TMA || (h->kernel == LBM_KERNEL_CELL && !odd_step(h)) || h->g.ny < 3) return false;
     const long long cells = (long long)h->g.nx * h->g.ny * h->g.nz;
-    if (h->precision == LBM_FP32 && h->layout == LBM_PULL2) return cells >= kSplitFp32Min && cells < kSplitFp32Max;
-    return true;
+    if (h->precision == LBM_FP16_SHIFTED) return true;
+    return h->layout == LBM_AA ? cells >= kSplitFp32AaMin : cells >= kSplitFp32Min && cells < kSplitFp32Max;
 }
 
 bool whole_even_step(const lbm_handle *h)
@@ -438,14 +442,26 @@ int launch_step(lbm_handle *h, cudaStream_t s, int src, bool stats, cudaStream_t
 }
 
 // Steps of the graphs that plain runs are made of. Long runs go in chunks from
-// phase 0, what is left in quarters of a chunk from either phase and single
+// phase 0, what is left in graphs of four steps from either phase and single
 // launches; a run that starts in phase 1 takes one single step first. So a run
 // of 10 steps (a monitoring interval, the head of a sampled run) no longer falls
 // to single launches, whose wall rows run behind the interior rows or at their
-// end: 10 steps of 256x64x128 FP32 AA take 478 us in place of 550. A graph costs
-// about 4 us a node to build once, so a chunk is 16 steps of one launch or 8 of two
-// (24 nodes in all; with 16 of two, the first call took 290 us against 130).
+// end. A graph costs about 4 us a node to build once, so a chunk is 16 steps of one
+// launch or 8 of two (24 and 32 nodes with the quarters); graphs of two steps
+// save less than their launch costs on small grids (3 steps of 64x32x32 FP32 AA
+// 26.6 us against 21.6).
+constexpr int kQuarterSteps = 4;
 int chunk_steps(const lbm_handle *h) { return split_step(h) ? 8 : 16; }
+
+// Whether what a chunk leaves over goes in quarters. One-launch steps that start
+// under programmatic dependent launch follow each other as closely outside a
+// graph as in one, and changing between the two costs 2 us.
+bool use_quarters(const lbm_handle *h)
+{
+    const bool pdl = (h->kernel == LBM_KERNEL_PAIR || h->kernel == LBM_KERNEL_QUAD) &&
+                     !(h->precision == LBM_FP32 && h->layout == LBM_PULL2);
+    return split_step(h) || !pdl;
+}
 
 // Graph of `steps` steps from lattice (or phase) start, the first one sampled
 // when `sample`.
@@ -497,9 +513,9 @@ int ensure_chunks(lbm_handle *h)
         const int rc = build_graph(h, 0, chunk_steps(h), false, &h->chunk);
         if (rc != LBM_OK) return rc;
     }
-    for (int start = 0; start < 2; ++start)
+    for (int start = 0; start < 2 && use_quarters(h); ++start)
         if (!h->quarter[start]) {
-            const int rc = build_graph(h, start, chunk_steps(h) / 4, false, &h->quarter[start]);
+            const int rc = build_graph(h, start, kQuarterSteps, false, &h->quarter[start]);
             if (rc != LBM_OK) return rc;
         }
     const int len = h->stats_every > 0 ? 1 + (h->stats_every - 1) % chunk_steps(h) : 0;
@@ -885,7 +901,8 @@ int lbm_step(lbm_handle *h, int n)
         const int rc = ensure_chunks(h);
         if (rc != LBM_OK) return rc;
     }
-    const int chunk = chunk_steps(h), quarter = chunk / 4;
+    const int chunk = chunk_steps(h);
+    const bool quarters = use_quarters(h);
     while (n > 0) {
         const bool sample = h->stats_every > 0 && (h->step % h->stats_every) == 0;
         if (sample && h->stats_every % chunk != 1 && n >= h->period_len) {
@@ -915,8 +932,8 @@ int lbm_step(lbm_handle *h, int n)
             if (h->cur == 0 && run >= chunk) {
                 done = chunk;
                 CK(cudaGraphLaunch(h->chunk, h->stream));
-            } else if (run >= quarter && run <= chunk) {
-                done = quarter;
+            } else if (quarters && run >= kQuarterSteps && run <= chunk) {
+                done = kQuarterSteps;
                 CK(cudaGraphLaunch(h->quarter[h->cur], h->stream));
             } else {
                 done = 1;

@@ -37,7 +37,7 @@ struct lbm_handle {
     int *err;                    // device flag set by a timed-out pipeline wait
     long long wait_limit;        // clock cycles a pipeline wait may take before it gives up
     cudaGraphExec_t chunk;       // plain steps starting from cur = 0 (chunk_steps in lbm.cu)
-    cudaGraphExec_t quarter[2];  // a quarter as many, starting from cur = 0 / 1
+    cudaGraphExec_t quarter[2];  // kQuarterSteps of them, starting from cur = 0 / 1
     cudaGraphExec_t period[2];   // a sampled step and the period_len - 1 plain ones after it, from cur = 0 / 1
     int period_len;
     bool member;                 // member view of a batch (stepped by the batch)

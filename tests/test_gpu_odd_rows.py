@@ -12,8 +12,9 @@ pytestmark = pytest.mark.gpu
 @pytest.mark.parametrize("mrt", [False, True])
 @pytest.mark.parametrize("layout", [lbm.PULL2, lbm.AA])
 @pytest.mark.parametrize("precision", [lbm.FP32, lbm.FP16_SHIFTED])
-@pytest.mark.parametrize("nx,ny,nz,wall", [(1, 5, 2, 1), (3, 2, 3, 0), (5, 3, 1, 2), (61, 6, 3, 1), (63, 5, 4, 0),
-                                           (65, 4, 3, 1), (127, 3, 3, 2), (129, 7, 2, 1), (257, 4, 3, 0), (255, 33, 40, 1)])
+@pytest.mark.parametrize("nx,ny,nz,wall", [  # 2^17 cells and more run two cells a thread, the last case does not
+    (1, 1024, 128, 1), (3, 2, 21846, 0), (5, 3, 8739, 2), (61, 43, 50, 1), (63, 46, 46, 0), (65, 64, 32, 1),
+    (127, 3, 345, 2), (129, 32, 32, 1), (257, 30, 17, 0), (255, 33, 40, 1), (31, 65, 65, 0)])
 def test_odd_rows_match_the_one_cell_kernel(nx, ny, nz, wall, precision, layout, mrt):
     case = workload.derive_channel("odd", nx, ny, nz, 640.0, wall=wall).with_(force=(2e-6, 1e-7, -1e-6))
     out = []
