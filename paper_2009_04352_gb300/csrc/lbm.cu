@@ -568,6 +568,26 @@ int export_state(lbm_handle *h, double *pops, double *part)
     return LBM_OK;
 }
 
+// Device staging of uploaded FP64 populations: the lattice that the next step will
+// overwrite, for as many directions at a time as it holds (9 in FP32, 4 in FP16
+// storage), or for the one lattice of AA a buffer of all 19 (*own). Mapping a whole
+// staging buffer on each call cost 0.8 of 2.8 ms at 256x64x128 (319 MB) and took 20
+// GB at 1024x256x512. (Downloads keep the one buffer: three pageable copies into
+// fresh pages are slower than one, 5.4 ms against 1.6 at 64x32x32.)
+int populations_staging(lbm_handle *h, double **d, int *directions, bool *own)
+{
+    const size_t n = (size_t)h->g.nx * h->g.ny * h->g.nz;
+    *own = h->layout == LBM_AA;
+    *directions = lbm::Q;
+    if (*own) {
+        if (cudaMallocAsync((void **)d, lbm::Q * n * sizeof(double), h->stream) == cudaSuccess) return LBM_OK;
+        return fail(LBM_ERR_OOM, "staging buffer");
+    }
+    *d = (double *)h->f[h->cur ^ 1];
+    *directions = (int)(lbm::Q * (size_t)h->g.plane * elem_size(h) / (n * sizeof(double)));
+    return LBM_OK;
+}
+
 // sum f - 1 and sum e f with FP64 additions per cell (any magnitude).
 int conservation_fp64(lbm_handle *h, double *out)
 {
@@ -853,19 +873,25 @@ int lbm_set_populations(lbm_handle *h, const double *host_in)
 {
     LbmRange range("lbm_set_populations");
     if (!h || !host_in) return fail(LBM_ERR_ARG, "NULL argument");
-    const size_t b = (size_t)lbm::Q * h->g.nx * h->g.ny * h->g.nz * sizeof(double);
+    const size_t n = (size_t)h->g.nx * h->g.ny * h->g.nz;
     double *d = nullptr;
-    if (cudaMallocAsync((void **)&d, b, h->stream) != cudaSuccess) return fail(LBM_ERR_OOM, "staging buffer");
-    CK(cudaMemcpyAsync(d, host_in, b, cudaMemcpyHostToDevice, h->stream));
+    int some = 0;
+    bool own = false;
+    const int rc = populations_staging(h, &d, &some, &own);
+    if (rc != LBM_OK) return rc;
     const dim3 grid = grid_of(h, 128);
     if (h->layout == LBM_AA) h->cur = 0;
     const int map = lbm_state_map(h);
-    if (h->precision == LBM_FP16_SHIFTED)
-        lbm::k_scatter<__half><<<grid, 128, 0, h->stream>>>(d, (__half *)lbm_state_ptr(h), h->g, h->p.wall, map);
-    else
-        lbm::k_scatter<float><<<grid, 128, 0, h->stream>>>(d, (float *)lbm_state_ptr(h), h->g, h->p.wall, map);
-    CK_LAUNCH();
-    CK(cudaFreeAsync(d, h->stream));
+    for (int a0 = 0; a0 < lbm::Q; a0 += some) {
+        const int a1 = std::min(a0 + some, lbm::Q);
+        CK(cudaMemcpyAsync(d, host_in + a0 * n, (a1 - a0) * n * sizeof(double), cudaMemcpyHostToDevice, h->stream));
+        if (h->precision == LBM_FP16_SHIFTED)
+            lbm::k_scatter<__half><<<grid, 128, 0, h->stream>>>(d, a0, a1, (__half *)lbm_state_ptr(h), h->g, h->p.wall, map);
+        else
+            lbm::k_scatter<float><<<grid, 128, 0, h->stream>>>(d, a0, a1, (float *)lbm_state_ptr(h), h->g, h->p.wall, map);
+        CK_LAUNCH();
+    }
+    if (own) CK(cudaFreeAsync(d, h->stream));
     CK(cudaStreamSynchronize(h->stream));
     h->step = 0;
     return LBM_OK;

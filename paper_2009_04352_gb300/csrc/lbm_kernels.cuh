@@ -575,11 +575,11 @@ template <typename T> __device__ __forceinline__ void st_d(T *p, double v);
 template <> __device__ __forceinline__ void st_d<float>(float *p, double v) { *p = __double2float_rn(v); }
 template <> __device__ __forceinline__ void st_d<__half>(__half *p, double v) { *p = __double2half(v); }
 
-// Write f_a(x) (FP64, unshifted, dense) into the slot that the gather of
-// (x, a) reads under storage map `map`, so that the next gather returns
-// exactly these populations.
+// Write f_a(x), a0 <= a < a1 (FP64, unshifted, dense), into the slot that the
+// gather of (x, a) reads under storage map `map`, so that the next gather
+// returns exactly these populations.
 template <typename T>
-__global__ void k_scatter(const double *__restrict__ in, T *__restrict__ dst, Geom g, int wall, int map)
+__global__ void k_scatter(const double *__restrict__ in, int a0, int a1, T *__restrict__ dst, Geom g, int wall, int map)
 {
     const int x = blockIdx.x * blockDim.x + threadIdx.x;
     const int y = blockIdx.y, z = blockIdx.z;
@@ -588,7 +588,9 @@ __global__ void k_scatter(const double *__restrict__ in, T *__restrict__ dst, Ge
     const long long ncell = (long long)g.nx * g.ny * g.nz;
     const long long cell = ((long long)z * g.ny + y) * g.nx + x;
 #pragma unroll
-    for (int a = 0; a < Q; ++a) st_d<T>(dst + state_offset(g, wall, map, a, x, y, z, n), in[a * ncell + cell] - w_of(a));
+    for (int a = 0; a < Q; ++a)
+        if (a >= a0 && a < a1)
+            st_d<T>(dst + state_offset(g, wall, map, a, x, y, z, n), in[(a - a0) * ncell + cell] - w_of(a));
 }
 
 // SplitMix64 (Steele, Lea & Flood 2014): first output for state s.
