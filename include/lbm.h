@@ -134,17 +134,17 @@ typedef enum {
 } lbm_layout;
 
 /* Form of the fused step kernel (all compute the same update).
- *   CELL: one thread per cell, any grid.
+ *   CELL: one thread per cell, any grid (plain steps on odd nx with halfway walls
+ *         and at least 2^17 cells run two cells per thread, the same bits).
  *   PAIR: two cells per thread, 2-wide loads and packed FP32 math; even nx.
  *   TMA:  two cells per thread; each CTA streams whole source rows into a
  *         shared-memory ring with bulk asynchronous copies (full/empty
  *         mbarriers, 2-4 stages); nx a multiple of 64 whose rows fit the ring.
  *   QUAD: four cells per thread, 8-byte loads and stores; FP16 storage and nx a
- *         multiple of 4. With the two-lattice layout and BGK (or wall nodes)
- *         a step is two launches, the interior rows and then the two wall
- *         rows, the latter with the two-cell tile (the same bits); with MRT
- *         and halfway walls one launch whose wall rows call a separately
- *         compiled four-cell wall tile.
+ *         multiple of 4.
+ * Inside the step graphs PAIR and QUAD steps mostly run as two parallel launches,
+ * the interior rows and the two wall rows, the latter with the two-cell tile (the
+ * same bits as the one-launch forms that single steps run).
  *   AUTO: QUAD where allowed, else PAIR for even nx, else CELL. */
 typedef enum {
     LBM_KERNEL_AUTO = 0,
@@ -204,7 +204,8 @@ int lbm_create_from_buffers(lbm_grid g, double tau, double C_s, const double for
 int lbm_init_channel(lbm_handle *h, const double *u_mean_x, double noise_amp, uint64_t seed);
 
 /* Replace the populations by host_in (FP64, [19][nz][ny][nx], not shifted).
- * Rounded once to the storage precision. Resets the step counter to 0. */
+ * Rounded once to the storage precision. Resets the step counter to 0. With
+ * PULL2 the copy is staged in the lattice that the next step overwrites. */
 int lbm_set_populations(lbm_handle *h, const double *host_in);
 
 /* Copy the current populations f_a(x, t) to host_out (FP64, [19][nz][ny][nx],
@@ -291,7 +292,8 @@ int lbm_plane_stats(lbm_handle *h, double *out, double *wall_out, long long *n_s
                     int reset);
 
 /* Global mass and raw momentum of the current populations, out[4] =
- * (sum f, sum e_x f, sum e_y f, sum e_z f), reduced in FP64 (host pointer;
+ * (sum f, sum e_x f, sum e_y f, sum e_z f), added in compensated FP32 runs and
+ * then in FP64, to about 2^-44 of the sum of magnitudes (host pointer;
  * synchronises). Returns LBM_ERR_DIVERGED if any sum is NaN or Inf. */
 int lbm_conservation(lbm_handle *h, double *out);
 
