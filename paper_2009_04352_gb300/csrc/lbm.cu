@@ -270,6 +270,16 @@ bool split_step(const lbm_handle *h)
     return h->layout == LBM_AA ? cells >= kSplitFp32AaMin : cells >= kSplitFp32Min && cells < kSplitFp32Max;
 }
 
+// Whether a plain one-launch FP32 two-lattice step of the two-cell kernel on stream
+// s reads coherently and starts under programmatic dependent launch: between
+// single launches on small grids the gap costs more than the read-only path
+// gives (us a step, read-only / dependent: 16x8x8 8.3 / 5.5, 130x20x20 8.4 / 6.0,
+// 64x32x32 8.4 / 7.1). Inside graphs it does not (64x32x32 4.4 / 4.8).
+bool dependent_launch(const lbm_handle *h, cudaStream_t s)
+{
+    return s == h->stream && h->kernel == LBM_KERNEL_PAIR && (long long)h->g.nx * h->g.ny * h->g.nz < kSplitFp32Min;
+}
+
 bool whole_even_step(const lbm_handle *h)
 {
     return h->kernel == LBM_KERNEL_QUAD && (long long)h->g.nx * h->g.ny * h->g.nz >= kWholeEvenCells;
@@ -364,6 +374,10 @@ cudaError_t launch_whole(lbm_handle *h, cudaStream_t s, const T *src, T *dst)
             }
         }
     }
+    if constexpr (LAY == lbm::LAY_PULL && lbm::pull_nc<T> && !STATS)
+        if (dependent_launch(h, s))
+            return launch_ex(true, lbm::k_step_pair<T, STATS, COLL, lbm::ROWS_ALL, false, false>, grid, block, 0, s, src, dst, h->g,
+                             h->p, h->tw, h->part);
     if constexpr (LAY == lbm::LAY_PULL)
         // read-only loads of the source lattice: no programmatic dependent launch
         return launch_ex(!lbm::pull_nc<T>, lbm::k_step_pair<T, STATS, COLL, lbm::ROWS_ALL, false>, grid, block, 0, s, src, dst,

@@ -179,7 +179,8 @@ __device__ __forceinline__ float row_smag(const Phys &p, int y, int ny)
 // step that read the previous step's output that way, launched while that step
 // drained, read stale populations). So the two-lattice FP32 kernels, whose
 // read-only loads measure faster, launch without programmatic dependent
-// launch, and every other step kernel, launched with it, reads through
+// launch (single launches on small grids take a coherent instantiation with it,
+// dependent_launch in lbm.cu), and every other step kernel, launched with it, reads through
 // explicitly coherent loads (ldc, ld.global.ca), which the compiler neither
 // turns into read-only loads nor moves above the wait.
 template <typename T> constexpr bool pull_nc = std::is_same<T, float>::value;

@@ -70,11 +70,11 @@ __device__ __forceinline__ float2 row_pair(const T *row, int x0, int nx, int lan
 // reads the pull map through the read-only path; LAY_AA_ODD reads the same
 // positions in the opposite slots (map MAP_AA1); LAY_AA_EVEN reads the own
 // slots (map MAP_AA0).
-template <typename T, int ROW, int LAY = LAY_PULL>
+template <typename T, int ROW, int LAY = LAY_PULL, bool READ_ONLY = pull_nc<T>>
 __device__ __forceinline__ void gather_pair(const T *src, const Geom &g, int wall, int x0, int y, int z, int zm,
                                             int zp, int lane, float2 (&f)[Q])
 {
-    constexpr bool NC = LAY == LAY_PULL && pull_nc<T>;
+    constexpr bool NC = LAY == LAY_PULL && READ_ONLY;
     if constexpr (LAY == LAY_AA_EVEN) {
         const T *own = src + ((long long)z * g.ny + y) * g.sx + x0;
 #pragma unroll
@@ -542,7 +542,8 @@ __device__ __forceinline__ PairState collide_pair(float2 (&f)[Q], const Phys &p,
 // LAY selects the storage scheme (LAY_PULL: src and dst are the two lattices;
 // LAY_AA_EVEN / LAY_AA_ODD: src == dst, the single AA array).
 // ROWS: the row set the instantiation serves (no wall-layer code for the interior rows).
-template <typename T, bool STATS, int COLL = COLL_BGK, int LAY = LAY_PULL, int ROWS = ROWS_ALL>
+// READ_ONLY: two-lattice sources go through the read-only path (pull_nc).
+template <typename T, bool STATS, int COLL = COLL_BGK, int LAY = LAY_PULL, int ROWS = ROWS_ALL, bool READ_ONLY = pull_nc<T>>
 __device__ __forceinline__ void pair_tile(const T *src, T *dst, const Geom &g, const Phys &p,
                                           float *__restrict__ tw_out, double *__restrict__ part_blk, int xb, int y,
                                           int z)
@@ -561,7 +562,7 @@ __device__ __forceinline__ void pair_tile(const T *src, T *dst, const Geom &g, c
     CellState ca0{}, ca1{};
     if (node_row) {
         float2 fa[Q];
-        gather_pair<T, ROW_INTERIOR, LAY>(src, g, p.wall, xl, y == 0 ? 1 : g.ny - 2, z, zm, zp, lane, fa);
+        gather_pair<T, ROW_INTERIOR, LAY, READ_ONLY>(src, g, p.wall, xl, y == 0 ? 1 : g.ny - 2, z, zm, zp, lane, fa);
         float a0[Q], a1[Q];
 #pragma unroll
         for (int a = 0; a < Q; ++a) {
@@ -574,11 +575,11 @@ __device__ __forceinline__ void pair_tile(const T *src, T *dst, const Geom &g, c
 
     float2 f[Q];
     if (ROWS != ROWS_INTERIOR && y == 0)
-        gather_pair<T, ROW_BOTTOM, LAY>(src, g, p.wall, xl, y, z, zm, zp, lane, f);
+        gather_pair<T, ROW_BOTTOM, LAY, READ_ONLY>(src, g, p.wall, xl, y, z, zm, zp, lane, f);
     else if (ROWS != ROWS_INTERIOR && y == g.ny - 1)
-        gather_pair<T, ROW_TOP, LAY>(src, g, p.wall, xl, y, z, zm, zp, lane, f);
+        gather_pair<T, ROW_TOP, LAY, READ_ONLY>(src, g, p.wall, xl, y, z, zm, zp, lane, f);
     else
-        gather_pair<T, ROW_INTERIOR, LAY>(src, g, p.wall, xl, y, z, zm, zp, lane, f);
+        gather_pair<T, ROW_INTERIOR, LAY, READ_ONLY>(src, g, p.wall, xl, y, z, zm, zp, lane, f);
 
     float2 twx = bc(0.f), twz = bc(0.f);
     PairState c;
@@ -663,7 +664,7 @@ __device__ __forceinline__ void pdl_begin()
 #define LBM_PAIR_MRT_MIN_BLOCKS 5   // the same for the MRT instantiations (96 registers)
 #endif
 
-template <typename T, bool STATS, int COLL, int ROWS, bool REV>
+template <typename T, bool STATS, int COLL, int ROWS, bool REV, bool READ_ONLY = pull_nc<T>>
 __global__ void __launch_bounds__(128, COLL == COLL_MRT ? LBM_PAIR_MRT_MIN_BLOCKS : LBM_PAIR_MIN_BLOCKS)
     k_step_pair(const T *__restrict__ src, T *__restrict__ dst, Geom g, Phys p, float *__restrict__ tw_out,
                 double *__restrict__ part)
@@ -672,8 +673,8 @@ __global__ void __launch_bounds__(128, COLL == COLL_MRT ? LBM_PAIR_MRT_MIN_BLOCK
     int y, z;
     row_of_block<ROWS, REV>(g, y, z);
     const long long blk = ((long long)y * g.nz + z) * gridDim.x + blockIdx.x;
-    pair_tile<T, STATS, COLL, LAY_PULL, ROWS>(src, dst, g, p, tw_out, STATS ? part + blk * K_PART : nullptr, blockIdx.x,
-                                              y, z);
+    pair_tile<T, STATS, COLL, LAY_PULL, ROWS, READ_ONLY>(src, dst, g, p, tw_out, STATS ? part + blk * K_PART : nullptr,
+                                                         blockIdx.x, y, z);
 }
 
 // The two wall rows of a step whose interior rows run in a launch of their
