@@ -212,15 +212,18 @@ __device__ __forceinline__ double block_sums(double (&v)[16])
 
 constexpr float VEL_SCALE = 1073741824.f;   // 2^30
 
+// Whether a cell's terms go to the FP32 sums: rho from 1/2, below which rho - 1
+// outweighs the density that its sum stands for, to 2^24, above which the 1 falls
+// between two FP32 numbers, and velocities whose products FP32 holds. False for NaN.
 __device__ __forceinline__ bool profile_in_range(float rho, float ux, float uy, float uz)
 {
-    return fmaf(fabsf(rho), 1e-6f, fabsf(ux) + fabsf(uy) + fabsf(uz)) < 1e6f;
+    return rho >= 0.5f && rho <= 16777216.f && fabsf(ux) + fabsf(uy) + fabsf(uz) < 1e6f;
 }
 
 __device__ __forceinline__ void profile_add_fp64(double (&v)[16], float rho, float fx, float fy, float fz)
 {
     const double r = rho, ux = fx, uy = fy, uz = fz;
-    v[0] += r - 1.0;
+    v[0] += r;
     v[1] += ux;
     v[2] += uy;
     v[3] += uz;
@@ -283,7 +286,6 @@ __global__ void __launch_bounds__(128, SUM_BLOCKS<T, PROFILE>) k_plane_sums(cons
         Cells<V> in;
         gather_cells<T, V, LAY>(src, g, p.wall, valid ? x0 : g.nx - V, y, z, lane, in);
         if (valid) {
-            cells += V;
 #pragma unroll
             for (int h = 0; h < NP; ++h) {
                 float2 f[Q];
@@ -295,7 +297,8 @@ __global__ void __launch_bounds__(128, SUM_BLOCKS<T, PROFILE>) k_plane_sums(cons
                         // velocities scaled by 2^30, so that the residuals of small squares stay normal
                         const float2 vx = mul2(c.ux, bc(VEL_SCALE)), vy = mul2(c.uy, bc(VEL_SCALE)),
                                      vz = mul2(c.uz, bc(VEL_SCALE));
-                        sum_add(s[0], sub2(c.rho, bc(1.f)));   // exact; the cell count is added below
+                        sum_add(s[0], sub2(c.rho, bc(1.f)));   // exact; the count of these cells is added below
+                        cells += V == 1 ? 1 : 2;
                         sum_add(s[1], c.ux);
                         sum_add(s[2], c.uy);
                         sum_add(s[3], c.uz);
@@ -306,7 +309,7 @@ __global__ void __launch_bounds__(128, SUM_BLOCKS<T, PROFILE>) k_plane_sums(cons
                         sum_mul(s[8], c.rho, c.ux);
                         sum_mul(s[9], c.rho, c.uy);
                         sum_mul(s[10], c.rho, c.uz);
-                    } else {   // a diverged cell: its products may overflow FP32
+                    } else {
                         profile_add_fp64(v, c.rho.x, c.ux.x, c.uy.x, c.uz.x);
                         if (V > 1) profile_add_fp64(v, c.rho.y, c.ux.y, c.uy.y, c.uz.y);
                     }
