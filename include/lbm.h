@@ -292,8 +292,8 @@ int lbm_plane_stats(lbm_handle *h, double *out, double *wall_out, long long *n_s
                     int reset);
 
 /* Global mass and raw momentum of the current populations, out[4] =
- * (sum f, sum e_x f, sum e_y f, sum e_z f), added in compensated FP32 runs and
- * then in FP64, to about 2^-44 of the sum of magnitudes (host pointer;
+ * (sum f, sum e_x f, sum e_y f, sum e_z f), to the accuracy of FP64 additions
+ * (error-free FP32 additions in short runs, then FP64; host pointer;
  * synchronises). Returns LBM_ERR_DIVERGED if any sum is NaN or Inf. */
 int lbm_conservation(lbm_handle *h, double *out);
 

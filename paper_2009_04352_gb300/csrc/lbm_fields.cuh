@@ -6,14 +6,18 @@
 // of k_export with FP64 sums did not: FP64 runs at 1/64 of the FP32 rate here, and
 // FP16 storage was read 2 bytes at a time. us a call at 512x128x256, before / now
 // (floor, the reads and writes at the copy rate): conservation FP32 3980 / 388 (188),
-// FP16 3967 / 266 (94); plane profile FP32 739 / 306, AA 721 / 218 (188), FP16 736 /
-// 214 (94); moments FP32 234 / 220 (228), FP16 206 / 158, AA 181 / 133 (134). Here a thread gathers V cells of a row with the wide loads of the
-// step kernels (gather_pair, gather_quad), and the sums run in compensated FP32:
+// AA 302, FP16 3967 / 300 (94), AA 229; plane profile FP32 739 / 320, AA 721 / 241 (188),
+// FP16 736 / 282 (94), AA 208; moments FP32 234 / 220 (228: a pass that mostly reads
+// can beat the copy rate), FP16 206 / 158, AA 181 / 133 (134).
+// Here a thread gathers V cells of a row with the wide loads of the step kernels
+// (gather_pair, gather_quad), and the sums run in FP32 without loss against FP64:
 // every addition is an error-free transformation (Knuth's two-sum; products with
-// their FMA residual), the residuals are added up beside it, and after at most
-// SUM_RUN additions the pair of sums is moved to FP64. A run's residual sum is
-// itself rounded to 2^-24 of at most SUM_RUN half ulps of the run's sum, about
-// 2^-46 of it, independently from run to run.
+// their FMA residual), its error is added to a second word error-free, and only the
+// errors of those additions to a third, with rounding. After n <= SUM_RUN cells the
+// three words move to FP64. With M the largest partial sum the second word stays
+// below 2 n 2^-24 M, the third below (2 n)^2 2^-48 M, so its roundings add up to less
+// than (2 n)^3 2^-72 M (2^-48 M for 128 cells, half the terms where a cell adds no
+// product); n additions in FP64 may lose n 2^-53 M, 2^-46 M.
 #pragma once
 
 #include <algorithm>
@@ -23,35 +27,50 @@
 
 namespace lbm {
 
-constexpr int SUM_RUN = 32;   // additions to one compensated sum before it goes to FP64
+constexpr int SUM_RUN = 128;   // cells in one compensated sum before it goes to FP64
 
-// Compensated sum of two lanes: hi + lo.
-struct Sum2 {
-    float2 hi, lo;
-};
-
-__device__ __forceinline__ void sum_add(Sum2 &s, float2 v)
+// a + b = s + e exactly, in both lanes.
+__device__ __forceinline__ float2 two_sum(float2 a, float2 b, float2 &e)
 {
-    const float2 t = add2(s.hi, v), b = sub2(t, s.hi);
-    s.lo = add2(s.lo, add2(sub2(s.hi, sub2(t, b)), sub2(v, b)));
-    s.hi = t;
+    const float2 s = add2(a, b), t = sub2(s, a);
+    e = add2(sub2(a, sub2(s, t)), sub2(b, t));
+    return s;
 }
 
-// s += a b with the product's rounding error
-__device__ __forceinline__ void sum_mul(Sum2 &s, float2 a, float2 b)
+// Two sums hi + mid + lo of FP32 terms, one a lane. mid takes the rounding
+// errors of hi and lo those of mid.
+struct Sum3 {
+    float2 hi, mid, lo;
+};
+
+__device__ __forceinline__ void sum_residual(Sum3 &s, float2 r)
+{
+    float2 e;
+    s.mid = two_sum(s.mid, r, e);
+    s.lo = add2(s.lo, e);
+}
+
+__device__ __forceinline__ void sum_add(Sum3 &s, float2 v)
+{
+    float2 e;
+    s.hi = two_sum(s.hi, v, e);
+    sum_residual(s, e);
+}
+
+// s += a b with the products' rounding errors
+__device__ __forceinline__ void sum_mul(Sum3 &s, float2 a, float2 b)
 {
     const float2 v = mul2(a, b);
-    s.lo = add2(s.lo, fma2(a, b, make_float2(-v.x, -v.y)));
+    sum_residual(s, fma2(a, b, make_float2(-v.x, -v.y)));
     sum_add(s, v);
 }
 
-// The sum over both lanes in FP64; clears s.
-__device__ __forceinline__ double sum_take(Sum2 &s)
+// Both sums in FP64; clears s.
+__device__ __forceinline__ double2 sum_take(Sum3 &s)
 {
-    const float t = __fadd_rn(s.hi.x, s.hi.y), b = __fsub_rn(t, s.hi.x);
-    const float e = __fadd_rn(__fsub_rn(s.hi.x, __fsub_rn(t, b)), __fsub_rn(s.hi.y, b));
-    const double v = (double)t + (double)__fadd_rn(e, __fadd_rn(s.lo.x, s.lo.y));
-    s.hi = s.lo = bc(0.f);
+    const double2 v = make_double2((double)s.hi.x + ((double)s.mid.x + (double)s.lo.x),
+                                   (double)s.hi.y + ((double)s.mid.y + (double)s.lo.y));
+    s.hi = s.mid = s.lo = bc(0.f);
     return v;
 }
 
@@ -214,10 +233,15 @@ constexpr float VEL_SCALE = 1073741824.f;   // 2^30
 
 // Whether a cell's terms go to the FP32 sums: rho from 1/2, below which rho - 1
 // outweighs the density that its sum stands for, to 2^24, above which the 1 falls
-// between two FP32 numbers, and velocities whose products FP32 holds. False for NaN.
+// between two FP32 numbers, and velocities whose products FP32 holds, and whose
+// products' errors it holds exactly: each 0 or at least 2^-81 (2^-51 scaled). False
+// for NaN.
 __device__ __forceinline__ bool profile_in_range(float rho, float ux, float uy, float uz)
 {
-    return rho >= 0.5f && rho <= 16777216.f && fabsf(ux) + fabsf(uy) + fabsf(uz) < 1e6f;
+    const float ax = fabsf(ux), ay = fabsf(uy), az = fabsf(uz);
+    // 0 wraps round to the largest word
+    const unsigned least = min(__float_as_uint(ax) - 1u, min(__float_as_uint(ay) - 1u, __float_as_uint(az) - 1u));
+    return rho >= 0.5f && rho <= 16777216.f && ax + ay + az < 1e6f && least >= ((127u - 81u) << 23) - 1u;
 }
 
 __device__ __forceinline__ void profile_add_fp64(double (&v)[16], float rho, float fx, float fy, float fz)
@@ -239,40 +263,50 @@ __device__ __forceinline__ void profile_add_fp64(double (&v)[16], float rho, flo
 // Sums over the row tiles blockIdx.x, blockIdx.x + gridDim.x, ... of plane
 // blockIdx.y (tile t: row z = t / nxb, cells from V blockDim (t % nxb)):
 //   PROFILE  rho, u, u_i^2, u_x u_y, rho u (K_STATS columns of lbm_plane_stats)
-//   else     sum of f - w and of e f (4 columns), one compensated sum for each
-//            direction, combined in FP64
-// to out[(y gridDim.x + blockIdx.x) columns]. The order of the additions depends
-// on the grid only, so every layout and storage map gives the same bits.
-// CTAs per SM the register budget must allow (us at 512x128x256, 3 / 4 / 5): FP32
-// profile 342 / 353 / 306, FP16 profile 222 / 214 / 235, conservation FP32 462 / 386 /
-// 415, FP16 262 / 265 / 364.
-template <typename T, bool PROFILE> constexpr int SUM_BLOCKS = PROFILE && sizeof(T) == 4 ? 5 : 4;
+//   else     sum of f - w and of e f (4 columns), one sum for each direction,
+//            combined in FP64
+// to out[(y gridDim.x + blockIdx.x) columns]. The two lanes of a sum hold two columns
+// (or opposite directions) of one cell, not one column of two cells: half the
+// registers for the same packed additions. The order of the additions depends on the
+// grid only, so every layout and storage map gives the same bits.
+// CTAs per SM the register budget must allow (us at 512x128x256 with sixteen CTAs an
+// SM in all, 3 / 4 / 5 / 6): FP32 profile 388 / 412 / 337 / 362, AA 232 / 235 / 258 /
+// 253, conservation 450 / 459 / 415 / 573, AA 315 / 294 / 328 / 450; FP16 profile 278 /
+// 283 / 300 / 304, conservation 302 / 299 / 340 / 400.
+template <typename T, int LAY> constexpr int SUM_BLOCKS = sizeof(T) == 4 && LAY == LAY_PULL ? 5 : 4;
 
 template <typename T, int V, int LAY, bool PROFILE>
-__global__ void __launch_bounds__(128, SUM_BLOCKS<T, PROFILE>) k_plane_sums(const T *__restrict__ src, Geom g, Phys p, int nxb,
-                                                       double *__restrict__ out)
+__global__ void __launch_bounds__(128, SUM_BLOCKS<T, LAY>) k_plane_sums(const T *__restrict__ src, Geom g, Phys p, int nxb,
+                                                                         double *__restrict__ out)
 {
-    constexpr int NP = (V + 1) / 2, NS = PROFILE ? K_STATS : Q, NOUT = PROFILE ? K_STATS : 4;
+    constexpr int NP = (V + 1) / 2, NS = PROFILE ? (K_STATS + 1) / 2 : (Q + 1) / 2, NOUT = PROFILE ? K_STATS : 4;
     const int lane = threadIdx.x & 31, y = blockIdx.y;
     const int tiles = nxb * g.nz;
-    Sum2 s[NS];
+    Sum3 s[NS];
 #pragma unroll
-    for (int k = 0; k < NS; ++k) s[k].hi = s[k].lo = bc(0.f);
+    for (int k = 0; k < NS; ++k) s[k].hi = s[k].mid = s[k].lo = bc(0.f);
     double v[16];
 #pragma unroll
     for (int k = 0; k < 16; ++k) v[k] = 0.0;
     auto take = [&]() {
         if constexpr (PROFILE) {
+            const double s1 = 1.0 / (double)VEL_SCALE, s2 = s1 * s1;
 #pragma unroll
-            for (int k = 0; k < NS; ++k)
-                v[k] += sum_take(s[k]) * (k >= 4 && k < 8 ? 1.0 / ((double)VEL_SCALE * VEL_SCALE) : 1.0);
+            for (int k = 0; k < NS; ++k) {
+                const double2 t = sum_take(s[k]);
+                const double scale = k < 2 ? 1.0 : (k < 4 ? s2 : s1);
+                v[2 * k] += t.x * scale;
+                if (2 * k + 1 < K_STATS) v[2 * k + 1] += t.y * scale;
+            }
         } else {
-            v[0] += sum_take(s[0]);
+            const double2 rest = sum_take(s[9]);
+            v[0] += rest.x + rest.y;
 #pragma unroll
             for (int k = 0; k < 9; ++k) {
                 const int a = 2 * k + 1;
-                const double va = sum_take(s[a]), vb = sum_take(s[a + 1]), d = va - vb;
-                v[0] += va + vb;
+                const double2 t = sum_take(s[k]);
+                const double d = t.x - t.y;
+                v[0] += t.x + t.y;
                 if (ex_of(a)) v[1] += ex_of(a) > 0 ? d : -d;
                 if (ey_of(a)) v[2] += ey_of(a) > 0 ? d : -d;
                 if (ez_of(a)) v[3] += ez_of(a) > 0 ? d : -d;
@@ -291,35 +325,38 @@ __global__ void __launch_bounds__(128, SUM_BLOCKS<T, PROFILE>) k_plane_sums(cons
                 float2 f[Q];
                 in.pair(h, f);
                 if constexpr (PROFILE) {
-                    PairState c = state_pair(f, p);
-                    if (V == 1) c.rho.y = 1.f, c.ux.y = c.uy.y = c.uz.y = 0.f;   // the unused lane adds nothing
-                    if (profile_in_range(c.rho.x, c.ux.x, c.uy.x, c.uz.x) && profile_in_range(c.rho.y, c.ux.y, c.uy.y, c.uz.y)) {
-                        // velocities scaled by 2^30, so that the residuals of small squares stay normal
-                        const float2 vx = mul2(c.ux, bc(VEL_SCALE)), vy = mul2(c.uy, bc(VEL_SCALE)),
-                                     vz = mul2(c.uz, bc(VEL_SCALE));
-                        sum_add(s[0], sub2(c.rho, bc(1.f)));   // exact; the count of these cells is added below
-                        cells += V == 1 ? 1 : 2;
-                        sum_add(s[1], c.ux);
-                        sum_add(s[2], c.uy);
-                        sum_add(s[3], c.uz);
-                        sum_mul(s[4], vx, vx);
-                        sum_mul(s[5], vy, vy);
-                        sum_mul(s[6], vz, vz);
-                        sum_mul(s[7], vx, vy);
-                        sum_mul(s[8], c.rho, c.ux);
-                        sum_mul(s[9], c.rho, c.uy);
-                        sum_mul(s[10], c.rho, c.uz);
-                    } else {
-                        profile_add_fp64(v, c.rho.x, c.ux.x, c.uy.x, c.uz.x);
-                        if (V > 1) profile_add_fp64(v, c.rho.y, c.ux.y, c.uy.y, c.uz.y);
+                    const PairState c = state_pair(f, p);
+#pragma unroll
+                    for (int l = 0; l < (V == 1 ? 1 : 2); ++l) {
+                        const float rho = l ? c.rho.y : c.rho.x, ux = l ? c.ux.y : c.ux.x, uy = l ? c.uy.y : c.uy.x,
+                                    uz = l ? c.uz.y : c.uz.x;
+                        if (profile_in_range(rho, ux, uy, uz)) {
+                            // velocities scaled by 2^30, so that the errors of small products stay normal
+                            const float2 vxy = make_float2(ux * VEL_SCALE, uy * VEL_SCALE);
+                            const float vz = uz * VEL_SCALE;
+                            sum_add(s[0], make_float2(__fsub_rn(rho, 1.f), ux));   // exact; these cells are counted in below
+                            ++cells;
+                            sum_add(s[1], make_float2(uy, uz));
+                            sum_mul(s[2], vxy, vxy);
+                            sum_mul(s[3], make_float2(vz, vxy.x), make_float2(vz, vxy.y));
+                            sum_mul(s[4], bc(rho), vxy);
+                            sum_mul(s[5], make_float2(rho, 0.f), make_float2(vz, 0.f));
+                        } else {
+                            profile_add_fp64(v, rho, ux, uy, uz);
+                        }
                     }
                 } else {
+                    sum_add(s[9], f[0]);
 #pragma unroll
-                    for (int a = 0; a < Q; ++a) sum_add(s[a], f[a]);
+                    for (int k = 0; k < 9; ++k) {
+                        sum_add(s[k], make_float2(f[2 * k + 1].x, f[2 * k + 2].x));
+                        if (V > 1) sum_add(s[k], make_float2(f[2 * k + 1].y, f[2 * k + 2].y));
+                    }
                 }
             }
         }
-        if (++run * NP >= SUM_RUN) {
+        run += V;
+        if (run + V > SUM_RUN) {
             take();
             run = 0;
         }
@@ -336,15 +373,18 @@ inline int cells_wide(const lbm_handle *h)
     return h->g.nx % 2 ? 1 : (h->precision == LBM_FP16_SHIFTED && h->g.nx % 4 == 0 ? 4 : 2);
 }
 
-// CTAs of k_plane_sums for each plane: about four rounds of the four CTAs an SM
-// holds of the 152 of this GPU over all planes, at most one for each row tile and
-// `most`. (More rounds shorten the runs between the FP64 sums, fewer leave SMs
-// idle at the end.)
+// CTAs of k_plane_sums for each plane: five rounds of the four CTAs an SM holds of
+// the 152 of this GPU over all planes (four of the five in two-lattice FP32), at most
+// one for each row tile and `most`. The number of SMs is written out, as the order of
+// the additions must not depend on the device. us at 512x128x256 with one / two /
+// three / four rounds of five: FP32 profile 439 / 352 / 327 / 320, conservation 529 /
+// 401 / 391 / 388; of four: FP16 profile 369 / 303 / 286 / 281, conservation 402 / 306 /
+// 297 / 296.
 inline int plane_sum_blocks(const lbm_handle *h, int most)
 {
     const int v = cells_wide(h), per_row = h->g.nx / v, bx = row_threads(per_row);
     const long long tiles = (long long)((per_row + bx - 1) / bx) * h->g.nz;
-    const int want = std::max(1, 4 * 4 * 152 / h->g.ny);
+    const int want = std::max(1, 5 * 4 * 152 / h->g.ny);
     return (int)std::min<long long>(std::min<long long>(want, most), tiles);
 }
 
