@@ -221,8 +221,9 @@ int lbm_set_stats_every(lbm_handle *h, int every);
  * from CUDA graphs of a few sizes (up to 16 steps). The first call with n > 0 after lbm_create,
  * lbm_set_kernel, lbm_set_les or lbm_set_wait_limit captures, instantiates and
  * uploads all of those graphs, whatever n is, so a
- * short warm-up call leaves nothing to build inside a later timed run; make
- * that first call outside any stream capture of the caller's own. With
+ * short warm-up call leaves nothing to build inside a later timed run. Inside a
+ * stream capture of the caller's own no graph is built or launched: every step
+ * is captured as launches of its own. With
  * sampling every k steps, a sampled step and the plain steps after it that do
  * not fill a graph are a graph too, built likewise on the first call after
  * lbm_set_stats_every changed k. */
@@ -357,7 +358,7 @@ long long lbm_batch_cells(lbm_batch *b);
  * `every` (0 = never), accumulated in each member's lbm_plane_stats. */
 int lbm_batch_set_stats_every(lbm_batch *b, int every);
 
-/* Advance every member by n steps. Asynchronous. */
+/* Advance every member by n steps. Asynchronous; graphs as for lbm_step. */
 int lbm_batch_step(lbm_batch *b, int n);
 
 /* Form of the batch step (no counterpart in the paper; both give every member

@@ -937,15 +937,16 @@ int lbm_step(lbm_handle *h, int n)
     LbmRange range("lbm_step");
     if (!h || n < 0) return fail(LBM_ERR_ARG, "invalid argument");
     if (h->member) return fail(LBM_ERR_STATE, "a batch member is advanced by lbm_batch_step");
-    if (n > 0) {
+    const bool graphs = n > 0 && !lbm_capturing(h->stream);
+    if (graphs) {
         const int rc = ensure_chunks(h);
         if (rc != LBM_OK) return rc;
     }
     const int chunk = chunk_steps(h);
-    const bool quarters = use_quarters(h);
+    const bool quarters = graphs && use_quarters(h);
     while (n > 0) {
         const bool sample = h->stats_every > 0 && (h->step % h->stats_every) == 0;
-        if (sample && h->stats_every % chunk != 1 && n >= h->period_len) {
+        if (graphs && sample && h->stats_every % chunk != 1 && n >= h->period_len) {
             CK(cudaGraphLaunch(h->period[h->cur], h->stream));
             h->nsamples += 1;
             h->cur ^= h->period_len & 1;
@@ -969,7 +970,7 @@ int lbm_step(lbm_handle *h, int n)
         }
         while (run > 0) {
             int done;
-            if (h->cur == 0 && run >= chunk) {
+            if (graphs && h->cur == 0 && run >= chunk) {
                 done = chunk;
                 CK(cudaGraphLaunch(h->chunk, h->stream));
             } else if (quarters && run >= kQuarterSteps && run <= chunk) {

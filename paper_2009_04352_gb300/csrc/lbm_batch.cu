@@ -475,7 +475,8 @@ int lbm_batch_step(lbm_batch *b, int n)
 {
     LbmRange range("lbm_batch_step");
     if (!b || n < 0) return fail(LBM_ERR_ARG, "invalid argument");
-    if (n > 0) {
+    const bool graphs = n > 0 && !lbm_capturing(b->stream);
+    if (graphs) {
         const int rc = ensure_chunks(b);
         if (rc != LBM_OK) return rc;
     }
@@ -494,15 +495,20 @@ int lbm_batch_step(lbm_batch *b, int n)
         if (b->stats_every > 0) run = std::min<long long>(run, b->stats_every - (b->step % b->stats_every));
         while (run > 0) {
             int done;
-            if (b->cur == 0 && run >= kBatchGraphSteps) {
+            if (graphs && b->cur == 0 && run >= kBatchGraphSteps) {
                 done = kBatchGraphSteps;
                 BK(cudaGraphLaunch(b->chunk, b->stream));
-            } else if (run >= kBatchQuarterSteps && run <= kBatchGraphSteps) {
+            } else if (graphs && run >= kBatchQuarterSteps && run <= kBatchGraphSteps) {
                 done = kBatchQuarterSteps;
                 BK(cudaGraphLaunch(b->quarter[b->cur], b->stream));
             } else {
                 done = 1;
-                BK(cudaGraphLaunch(b->one[b->cur], b->stream));
+                if (graphs) {
+                    BK(cudaGraphLaunch(b->one[b->cur], b->stream));
+                } else {
+                    const int rc = launch(b, b->stream, b->cur, false);
+                    if (rc != LBM_OK) return rc;
+                }
                 b->cur ^= 1;
             }
             b->step += done;

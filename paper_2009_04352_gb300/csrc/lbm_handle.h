@@ -57,6 +57,17 @@ inline int row_threads(int per_row)
     return 32 * ((warps + tiles - 1) / tiles);
 }
 
+// Whether the caller is capturing stream s. An executable graph can neither be
+// launched into a capture nor uploaded to its stream, so steps are single launches
+// then. (An error means that another stream's capture forbids the legacy stream.)
+inline bool lbm_capturing(cudaStream_t s)
+{
+    cudaStreamCaptureStatus status = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(s, &status) == cudaSuccess) return status != cudaStreamCaptureStatusNone;
+    cudaGetLastError();
+    return true;
+}
+
 // The array holding the current state and the map under which f(t) is stored.
 inline void *lbm_state_ptr(const lbm_handle *h) { return h->layout == LBM_AA ? h->f[0] : h->f[h->cur]; }
 inline int lbm_state_map(const lbm_handle *h)

@@ -54,13 +54,15 @@ def test_steps_in_a_capture(nx, ny, nz, precision, layout, every):
     b.close()
 
 
+@pytest.mark.parametrize("form", [lbm.BATCH_PERSISTENT, lbm.BATCH_MEMBER_GRIDS])
 @pytest.mark.parametrize("precision", [lbm.FP32, lbm.FP16_SHIFTED])
 @pytest.mark.parametrize("every", [0, 5])
-def test_batch_steps_in_a_capture(every, precision):
+def test_batch_steps_in_a_capture(every, precision, form):
     cases = [workload.derive_channel(f"m{i}", *s, 640.0) for i, s in enumerate(((32, 8, 16), (48, 12, 10), (64, 16, 32)))]
     stream, graph = torch.cuda.Stream(), torch.cuda.CUDAGraph()
     a, b = lbm.Batch(cases, precision=precision, stream=stream.cuda_stream), lbm.Batch(cases, precision=precision)
     for batch in (a, b):
+        batch.set_form(form)
         for m, c in zip(batch.members, cases):
             _start(m, c)
         batch.set_stats_every(3)
