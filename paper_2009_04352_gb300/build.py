@@ -11,7 +11,7 @@ CSRC = os.path.join(HERE, "csrc")
 BUILD = os.path.join(HERE, "_build")
 LIB = os.path.join(BUILD, "liblbm.so")
 SOURCES = ["lbm.cu", "lbm_noalloc.cu", "lbm_batch.cu"]
-HEADERS = ["lbm_device.cuh", "lbm_kernels.cuh", "lbm_pair.cuh", "lbm_tma.cuh", "lbm_handle.h", "lbm_quad.cuh", "lbm_fields.cuh", "lbm_odd.cuh"]
+HEADERS = ["lbm_device.cuh", "lbm_kernels.cuh", "lbm_pair.cuh", "lbm_tma.cuh", "lbm_handle.h", "lbm_graph_slot.h", "lbm_quad.cuh", "lbm_fields.cuh", "lbm_odd.cuh"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 
 

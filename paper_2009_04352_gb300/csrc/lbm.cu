@@ -59,11 +59,8 @@ int configure_rows(lbm_handle *h);
 
 void drop_graphs(lbm_handle *h)
 {
-    for (cudaGraphExec_t *g : {&h->chunk, &h->quarter[0], &h->quarter[1], &h->period[0], &h->period[1]})
-        if (*g) {
-            cudaGraphExecDestroy(*g);
-            *g = nullptr;
-        }
+    for (StepGraph *g : {&h->chunk, &h->quarter[0], &h->quarter[1], &h->period[0], &h->period[1]})
+        lbm::slot_clear(*g, cudaGraphExecDestroy);
 }
 
 int select_kernel(lbm_handle *h, int kernel)
@@ -477,8 +474,12 @@ bool use_quarters(const lbm_handle *h)
     return split_step(h) || !pdl;
 }
 
+// Steps of the graph of a sampled step and the plain ones after it that do not fill
+// a chunk; 1 where all of them do, 0 without sampling.
+int period_steps(const lbm_handle *h) { return h->stats_every > 0 ? 1 + (h->stats_every - 1) % chunk_steps(h) : 0; }
+
 // Graph of `steps` steps from lattice (or phase) start, the first one sampled
-// when `sample`.
+// when `sample`. After an error *out may hold a graph that was not uploaded.
 int build_graph(lbm_handle *h, int start, int steps, bool sample, cudaGraphExec_t *out)
 {
     cudaGraph_t graph = nullptr;
@@ -508,6 +509,7 @@ int build_graph(lbm_handle *h, int start, int steps, bool sample, cudaGraphExec_
     if (e != cudaSuccess) return fail(LBM_ERR_CUDA, "graph capture: %s", cudaGetErrorString(e));
     e = cudaGraphInstantiate(out, graph, 0);
     cudaGraphDestroy(graph);
+    if (e != cudaSuccess) *out = nullptr;
     if (e != cudaSuccess) return fail(LBM_ERR_CUDA, "graph instantiate: %s", cudaGetErrorString(e));
     // move the graph's device-side set-up off its first launch
     e = cudaGraphUpload(*out, h->stream);
@@ -523,29 +525,18 @@ int build_graph(lbm_handle *h, int start, int steps, bool sample, cudaGraphExec_
 // 252x80x126 MRT every plain step then ran as a single launch, 70 us against 66).
 int ensure_chunks(lbm_handle *h)
 {
-    if (!h->chunk) {
-        const int rc = build_graph(h, 0, chunk_steps(h), false, &h->chunk);
-        if (rc != LBM_OK) return rc;
-    }
-    for (int start = 0; start < 2 && use_quarters(h); ++start)
-        if (!h->quarter[start]) {
-            const int rc = build_graph(h, start, kQuarterSteps, false, &h->quarter[start]);
-            if (rc != LBM_OK) return rc;
-        }
-    const int len = h->stats_every > 0 ? 1 + (h->stats_every - 1) % chunk_steps(h) : 0;
-    if (len < 2) return LBM_OK;
-    for (int start = 0; start < 2; ++start) {
-        if (h->period[start] && h->period_len == len) continue;
-        if (h->period[start]) {
-            CK(cudaStreamSynchronize(h->stream));   // it may be in flight
-            cudaGraphExecDestroy(h->period[start]);
-            h->period[start] = nullptr;
-        }
-        const int rc = build_graph(h, start, len, true, &h->period[start]);
-        if (rc != LBM_OK) return rc;
-        if (start == 1) h->period_len = len;
-    }
-    return LBM_OK;
+    auto ensure = [h](StepGraph &g, int start, int steps, bool sample) {
+        // a graph of another length may be in flight
+        if (g.exec && g.steps != steps) CK(cudaStreamSynchronize(h->stream));
+        return lbm::slot_ensure(g, steps, cudaGraphExecDestroy,
+                                [=](cudaGraphExec_t *out) { return build_graph(h, start, steps, sample, out); });
+    };
+    int rc = ensure(h->chunk, 0, chunk_steps(h), false);
+    for (int start = 0; start < 2 && rc == LBM_OK && use_quarters(h); ++start)
+        rc = ensure(h->quarter[start], start, kQuarterSteps, false);
+    const int len = period_steps(h);
+    for (int start = 0; start < 2 && rc == LBM_OK && len > 1; ++start) rc = ensure(h->period[start], start, len, true);
+    return rc;
 }
 
 int ensure_part(lbm_handle *h, long long len)
@@ -942,16 +933,16 @@ int lbm_step(lbm_handle *h, int n)
         const int rc = ensure_chunks(h);
         if (rc != LBM_OK) return rc;
     }
-    const int chunk = chunk_steps(h);
+    const int chunk = chunk_steps(h), period = period_steps(h);
     const bool quarters = graphs && use_quarters(h);
     while (n > 0) {
         const bool sample = h->stats_every > 0 && (h->step % h->stats_every) == 0;
-        if (graphs && sample && h->stats_every % chunk != 1 && n >= h->period_len) {
-            CK(cudaGraphLaunch(h->period[h->cur], h->stream));
+        if (graphs && sample && period > 1 && n >= period) {
+            CK(cudaGraphLaunch(h->period[h->cur].exec, h->stream));
             h->nsamples += 1;
-            h->cur ^= h->period_len & 1;
-            h->step += h->period_len;
-            n -= h->period_len;
+            h->cur ^= period & 1;
+            h->step += period;
+            n -= period;
             continue;
         }
         if (sample) {
@@ -972,10 +963,10 @@ int lbm_step(lbm_handle *h, int n)
             int done;
             if (graphs && h->cur == 0 && run >= chunk) {
                 done = chunk;
-                CK(cudaGraphLaunch(h->chunk, h->stream));
+                CK(cudaGraphLaunch(h->chunk.exec, h->stream));
             } else if (quarters && run >= kQuarterSteps && run <= chunk) {
                 done = kQuarterSteps;
-                CK(cudaGraphLaunch(h->quarter[h->cur], h->stream));
+                CK(cudaGraphLaunch(h->quarter[h->cur].exec, h->stream));
             } else {
                 done = 1;
                 const int rc = launch_step(h, h->stream, h->cur, false);

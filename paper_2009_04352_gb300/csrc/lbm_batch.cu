@@ -159,7 +159,7 @@ struct lbm_batch {
     int cur;
     long long step;
     int stats_every;
-    cudaGraphExec_t chunk, quarter[2], one[2];
+    StepGraph chunk, quarter[2], one[2];
 };
 
 namespace {
@@ -168,11 +168,8 @@ size_t elem_bytes(int precision) { return precision == LBM_FP16_SHIFTED ? 2 : 4;
 
 void drop_graphs(lbm_batch *b)
 {
-    for (cudaGraphExec_t *g : {&b->chunk, &b->quarter[0], &b->quarter[1], &b->one[0], &b->one[1]})
-        if (*g) {
-            cudaGraphExecDestroy(*g);
-            *g = nullptr;
-        }
+    for (StepGraph *g : {&b->chunk, &b->quarter[0], &b->quarter[1], &b->one[0], &b->one[1]})
+        lbm::slot_clear(*g, cudaGraphExecDestroy);
 }
 
 template <typename T, int COLL>
@@ -301,7 +298,8 @@ int launch(lbm_batch *b, cudaStream_t s, int cur, bool stats)
     return LBM_OK;
 }
 
-// Graph of `steps` plain steps of all members from lattice start.
+// Graph of `steps` plain steps of all members from lattice start. After an error
+// *out may hold a graph that was not uploaded.
 int build_graph(lbm_batch *b, int start, int steps, cudaGraphExec_t *out)
 {
     cudaGraph_t graph = nullptr;
@@ -334,6 +332,7 @@ int build_graph(lbm_batch *b, int start, int steps, cudaGraphExec_t *out)
     if (e != cudaSuccess) return fail_cuda(e, "graph capture");
     e = cudaGraphInstantiate(out, graph, 0);
     cudaGraphDestroy(graph);
+    if (e != cudaSuccess) *out = nullptr;
     if (e != cudaSuccess) return fail_cuda(e, "graph instantiate");
     e = cudaGraphUpload(*out, b->stream);
     if (e != cudaSuccess) return fail_cuda(e, "graph upload");
@@ -344,11 +343,14 @@ int build_graph(lbm_batch *b, int start, int steps, cudaGraphExec_t *out)
 // its step count), so that no capture lands inside a later run.
 int ensure_chunks(lbm_batch *b)
 {
-    int rc = LBM_OK;
-    if (!b->chunk) rc = build_graph(b, 0, kBatchGraphSteps, &b->chunk);
+    auto ensure = [b](StepGraph &g, int start, int steps) {
+        return lbm::slot_ensure(g, steps, cudaGraphExecDestroy,
+                                [=](cudaGraphExec_t *out) { return build_graph(b, start, steps, out); });
+    };
+    int rc = ensure(b->chunk, 0, kBatchGraphSteps);
     for (int start = 0; start < 2 && rc == LBM_OK; ++start) {
-        if (!b->quarter[start]) rc = build_graph(b, start, kBatchQuarterSteps, &b->quarter[start]);
-        if (rc == LBM_OK && !b->one[start]) rc = build_graph(b, start, 1, &b->one[start]);
+        rc = ensure(b->quarter[start], start, kBatchQuarterSteps);
+        if (rc == LBM_OK) rc = ensure(b->one[start], start, 1);
     }
     return rc;
 }
@@ -379,7 +381,7 @@ int lbm_batch_create(int n, const lbm_member *members, int precision, void *cuda
     b->n = n;
     b->precision = precision;
     b->stream = (cudaStream_t)cuda_stream;
-    b->chunk = b->quarter[0] = b->quarter[1] = b->one[0] = b->one[1] = nullptr;
+    b->chunk = b->quarter[0] = b->quarter[1] = b->one[0] = b->one[1] = StepGraph{};
     b->pool = nullptr;
     b->d_inst = nullptr;
     b->cap = nullptr;
@@ -497,14 +499,14 @@ int lbm_batch_step(lbm_batch *b, int n)
             int done;
             if (graphs && b->cur == 0 && run >= kBatchGraphSteps) {
                 done = kBatchGraphSteps;
-                BK(cudaGraphLaunch(b->chunk, b->stream));
+                BK(cudaGraphLaunch(b->chunk.exec, b->stream));
             } else if (graphs && run >= kBatchQuarterSteps && run <= kBatchGraphSteps) {
                 done = kBatchQuarterSteps;
-                BK(cudaGraphLaunch(b->quarter[b->cur], b->stream));
+                BK(cudaGraphLaunch(b->quarter[b->cur].exec, b->stream));
             } else {
                 done = 1;
                 if (graphs) {
-                    BK(cudaGraphLaunch(b->one[b->cur], b->stream));
+                    BK(cudaGraphLaunch(b->one[b->cur].exec, b->stream));
                 } else {
                     const int rc = launch(b, b->stream, b->cur, false);
                     if (rc != LBM_OK) return rc;

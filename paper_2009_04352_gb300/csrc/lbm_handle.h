@@ -7,6 +7,9 @@
 
 #include "lbm.h"
 #include "lbm_device.cuh"
+#include "lbm_graph_slot.h"
+
+using StepGraph = lbm::GraphSlot<cudaGraphExec_t>;
 
 struct lbm_handle {
     lbm::Geom g;
@@ -36,10 +39,9 @@ struct lbm_handle {
     bool reverse;                // steps from lattice or phase 1 walk the planes backwards
     int *err;                    // device flag set by a timed-out pipeline wait
     long long wait_limit;        // clock cycles a pipeline wait may take before it gives up
-    cudaGraphExec_t chunk;       // plain steps starting from cur = 0 (chunk_steps in lbm.cu)
-    cudaGraphExec_t quarter[2];  // kQuarterSteps of them, starting from cur = 0 / 1
-    cudaGraphExec_t period[2];   // a sampled step and the period_len - 1 plain ones after it, from cur = 0 / 1
-    int period_len;
+    StepGraph chunk;             // plain steps starting from cur = 0 (chunk_steps in lbm.cu)
+    StepGraph quarter[2];        // kQuarterSteps of them, starting from cur = 0 / 1
+    StepGraph period[2];         // a sampled step and plain ones after it (period_steps), from cur = 0 / 1
     bool member;                 // member view of a batch (stepped by the batch)
     bool borrowed;               // population arrays owned by the caller or a batch, not freed here
     double nu_wall;              // viscosity of the wall law and of the van Driest y+
