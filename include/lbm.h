@@ -225,7 +225,7 @@ int lbm_set_stats_every(lbm_handle *h, int every);
  * stream capture of the caller's own no graph is built or launched: every step
  * is captured as launches of its own. With
  * sampling every k steps, a sampled step and the plain steps after it that do
- * not fill a graph are a graph too, built likewise on the first call after
+ * not fill a graph are a graph too, built on the first call with n > 1 after
  * lbm_set_stats_every changed k. */
 int lbm_step(lbm_handle *h, int n);
 

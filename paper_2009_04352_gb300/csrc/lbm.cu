@@ -520,10 +520,10 @@ int build_graph(lbm_handle *h, int start, int steps, bool sample, cudaGraphExec_
 // The graphs of plain steps, built together on the first step call after any
 // change that invalidated them, whatever the step count, so that no capture or
 // instantiation falls inside a later, longer run of steps. With
-// sampling, also the graphs of a sampled step and the plain steps after it that
+// sampling and n > 1, also the graphs of a sampled step and the plain steps after it that
 // do not fill a chunk (an interval of 10 would otherwise never reach one: of
 // 252x80x126 MRT every plain step then ran as a single launch, 70 us against 66).
-int ensure_chunks(lbm_handle *h)
+int ensure_chunks(lbm_handle *h, int n)
 {
     auto ensure = [h](StepGraph &g, int start, int steps, bool sample) {
         // a graph of another length may be in flight
@@ -535,7 +535,8 @@ int ensure_chunks(lbm_handle *h)
     for (int start = 0; start < 2 && rc == LBM_OK && use_quarters(h); ++start)
         rc = ensure(h->quarter[start], start, kQuarterSteps, false);
     const int len = period_steps(h);
-    for (int start = 0; start < 2 && rc == LBM_OK && len > 1; ++start) rc = ensure(h->period[start], start, len, true);
+    for (int start = 0; start < 2 && rc == LBM_OK && len > 1; ++start)
+        if (lbm::sampled_graph_due(n, h->stats_every, h->step, h->cur, start)) rc = ensure(h->period[start], start, len, true);
     return rc;
 }
 
@@ -930,14 +931,14 @@ int lbm_step(lbm_handle *h, int n)
     if (h->member) return fail(LBM_ERR_STATE, "a batch member is advanced by lbm_batch_step");
     const bool graphs = n > 0 && !lbm_capturing(h->stream);
     if (graphs) {
-        const int rc = ensure_chunks(h);
+        const int rc = ensure_chunks(h, n);
         if (rc != LBM_OK) return rc;
     }
     const int chunk = chunk_steps(h), period = period_steps(h);
     const bool quarters = graphs && use_quarters(h);
     while (n > 0) {
         const bool sample = h->stats_every > 0 && (h->step % h->stats_every) == 0;
-        if (graphs && sample && period > 1 && n >= period) {
+        if (graphs && sample && period > 1 && n >= period && h->period[h->cur].steps == period) {
             CK(cudaGraphLaunch(h->period[h->cur].exec, h->stream));
             h->nsamples += 1;
             h->cur ^= period & 1;

@@ -1,5 +1,6 @@
-// An executable graph kept together with the number of steps it advances, so that
-// a graph of another length is never taken for it. Host code without CUDA types.
+// Step graphs kept between calls: an executable graph together with the number of
+// steps it advances, so that a graph of another length is never taken for it, and
+// when one is worth building. Host code without CUDA types.
 #pragma once
 
 namespace lbm {
@@ -32,6 +33,17 @@ int slot_ensure(GraphSlot<Exec> &s, int steps, Destroy destroy, Build build)
     s.exec = e;
     s.steps = steps;
     return 0;
+}
+
+// Whether a call of n steps (or one after it) may replay a sampled step's graph from
+// phase `start`: sampling every `every` steps, at step `step` and phase `cur` now. An
+// even interval samples in one phase only. Calls of one step never replay one, and
+// callers that make nothing else need not pay for it.
+inline bool sampled_graph_due(int n, int every, long long step, int cur, int start)
+{
+    if (n < 2 || every < 2) return false;
+    const long long to_next = (every - step % every) % every;
+    return every % 2 || start == (cur ^ (int)(to_next & 1));
 }
 
 }  // namespace lbm

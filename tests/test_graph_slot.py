@@ -1,6 +1,7 @@
 """The step graphs kept between calls (lbm_graph_slot.h), compiled for the host with a
 fake of the graph: a slot never holds a graph of another length than it says, nor
-one whose building failed, whatever fails in between."""
+one whose building failed, whatever fails in between; and the graphs of sampled
+steps are built where a run replays them, not for calls of one step."""
 import subprocess
 
 from paper_2009_04352_gb300 import build
@@ -61,9 +62,41 @@ int main()
 }
 """
 
+DUE = r"""
+#include <cassert>
+#include "lbm_graph_slot.h"
 
-def test_slots_hold_what_they_say(tmp_path):
+int main()
+{
+    for (int every = 1; every <= 40; ++every)
+        for (long long step = 0; step <= 3 * every; ++step)
+            for (int cur = 0; cur < 2; ++cur) {
+                // phases in which the next samples fall, one plain or sampled step at a time
+                bool phase[2] = {false, false};
+                for (long long t = step; t <= step + 2 * every; ++t)
+                    if (t % every == 0) phase[cur ^ ((t - step) & 1)] = true;
+                for (int start = 0; start < 2; ++start) {
+                    assert(!lbm::sampled_graph_due(1, every, step, cur, start));
+                    const bool due = lbm::sampled_graph_due(2, every, step, cur, start);
+                    assert(due == lbm::sampled_graph_due(1000, every, step, cur, start));
+                    assert(due == (every > 1 && phase[start]));
+                }
+            }
+    return 0;
+}
+"""
+
+
+def _run(tmp_path, source):
     src, exe = tmp_path / "slot.cpp", tmp_path / "slot"
-    src.write_text(SOURCE)
+    src.write_text(source)
     subprocess.run(["g++", "-std=c++17", "-Wall", "-Werror", "-I" + build.CSRC, "-o", str(exe), str(src)], check=True)
     subprocess.run([str(exe)], check=True)
+
+
+def test_slots_hold_what_they_say(tmp_path):
+    _run(tmp_path, SOURCE)
+
+
+def test_sampled_graphs_are_built_where_they_are_replayed(tmp_path):
+    _run(tmp_path, DUE)
