@@ -13,6 +13,10 @@ LIB = os.path.join(BUILD, "liblbm.so")
 SOURCES = ["lbm.cu", "lbm_noalloc.cu", "lbm_batch.cu"]
 HEADERS = ["lbm_device.cuh", "lbm_kernels.cuh", "lbm_pair.cuh", "lbm_tma.cuh", "lbm_handle.h", "lbm_graph_slot.h", "lbm_quad.cuh", "lbm_fields.cuh", "lbm_odd.cuh"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
+# approximate FP32 division and square root (2 ulp): the relaxation time and
+# velocity tolerate it, and IEEE-exact forms cost ~4x the instructions
+FLAGS = [*ARCH, "-O3", "-lineinfo", "-std=c++17", "-prec-div=false", "-prec-sqrt=false",
+         "-Xcompiler", "-fPIC", "-I" + os.path.join(ROOT, "include")]
 
 
 def nvcc() -> str:
@@ -35,10 +39,7 @@ def build(force: bool = False, verbose: bool = False) -> str:
     if not force and not _stale(LIB, deps):
         return LIB
     tmp = LIB + f".tmp{os.getpid()}"
-    # approximate FP32 division and square root (2 ulp): the relaxation time and
-    # velocity tolerate it, and IEEE-exact forms cost ~4x the instructions
-    flags = [*ARCH, "-O3", "-lineinfo", "-std=c++17", "-prec-div=false", "-prec-sqrt=false",
-             "-Xcompiler", "-fPIC", "-I" + os.path.join(ROOT, "include")]
+    flags = list(FLAGS)
     if verbose:
         flags.append("-Xptxas=-v")
     objs = [os.path.join(BUILD, os.path.splitext(os.path.basename(s))[0] + f".{os.getpid()}.o") for s in srcs]

@@ -185,12 +185,15 @@ __device__ __forceinline__ float row_smag(const Phys &p, int y, int ny)
 // turns into read-only loads nor moves above the wait.
 template <typename T> constexpr bool pull_nc = std::is_same<T, float>::value;
 
-// Approximate division and square root of the collisions. The operands are
-// densities, relaxation times and stress norms, all normal numbers (or 0), for
-// which these single instructions give the bits of the full-range forms
-// (compared over every FP32 divisor from 1e-37 to 1e30); those carry scaling
-// code for subnormal and huge operands, about six instructions each, four of
-// them per cell. FULL keeps the full-range forms (the same bits).
+// Approximate division and square root of the collisions and of Spalding's law.
+// The operands are densities, relaxation times and stress norms. Where operands and
+// quotient are normal numbers (or 0) these single instructions give the bits of the
+// full-range forms; those carry scaling code for subnormal and huge operands, about
+// six instructions each, four of them per cell. A subnormal density deviation,
+// stress norm or Newton residual counts as 0 here, which changes no result: it is
+// added to a number at least 2^25 times as large. A density from 2^126 up, which no
+// state that has not diverged holds, gives 1/rho - 1 = 0 in place of -1. FULL keeps
+// the full-range forms.
 template <bool FULL> __device__ __forceinline__ float div_cell(float a, float b)
 {
     if (FULL) return a / b;
@@ -398,22 +401,33 @@ __device__ __forceinline__ Moments moments_of(const float (&f)[Q])
 // own relative step is below 1e-7, so a cell's result does not depend on which
 // cells share its warp (every kernel form gives the same bits); the warp
 // leaves the loop when all its lanes have stopped.
+__device__ __forceinline__ float spalding_start(float R, const Phys &p)
+{
+    const float up = sqrtf(R);
+    return R > 100.f ? fminf(up, __fadd_rn(logf(R) / p.kappa, p.B)) : up;
+}
+
+// One Newton step for a lane: u+ and whether it has stopped.
+__device__ __forceinline__ void spalding_step(float R, const Phys &p, float &up, bool &done)
+{
+    const float k = p.kappa * up;
+    const float ek = expf(k);
+    const float k2 = __fmul_rn(k, k);
+    const float t2 = __fsub_rn(__fsub_rn(__fsub_rn(ek, 1.f), k), __fmul_rn(0.5f, k2));   // e^k - 1 - k - k^2/2
+    const float t3 = __fsub_rn(t2, __fmul_rn(__fmul_rn(k2, k), 1.f / 6.f));            // ... - k^3/6
+    const float S = __fmaf_rn(p.ekb, t3, up);                                           // y+(u+)
+    const float dS = __fmaf_rn(__fmul_rn(p.ekb, p.kappa), t2, 1.f);                     // dy+/du+
+    const float step = done ? 0.f : div_cell<false>(__fmaf_rn(up, S, -R), __fmaf_rn(up, dS, S));
+    up -= step;
+    done = done || fabsf(step) <= 1e-7f * up;
+}
+
 __device__ __forceinline__ float spalding_uplus(float R, const Phys &p, unsigned mask)
 {
-    float up = sqrtf(R);
-    if (R > 100.f) up = fminf(up, __fadd_rn(logf(R) / p.kappa, p.B));
+    float up = spalding_start(R, p);
     bool done = false;
     for (int it = 0; it < p.newton_iters; ++it) {
-        const float k = p.kappa * up;
-        const float ek = expf(k);
-        const float k2 = __fmul_rn(k, k);
-        const float t2 = __fsub_rn(__fsub_rn(__fsub_rn(ek, 1.f), k), __fmul_rn(0.5f, k2));   // e^k - 1 - k - k^2/2
-        const float t3 = __fsub_rn(t2, __fmul_rn(__fmul_rn(k2, k), 1.f / 6.f));            // ... - k^3/6
-        const float S = __fmaf_rn(p.ekb, t3, up);                                           // y+(u+)
-        const float dS = __fmaf_rn(__fmul_rn(p.ekb, p.kappa), t2, 1.f);                     // dy+/du+
-        const float step = done ? 0.f : __fmaf_rn(up, S, -R) / __fmaf_rn(up, dS, S);
-        up -= step;
-        done = done || fabsf(step) <= 1e-7f * up;
+        spalding_step(R, p, up, done);
         if (__all_sync(mask, done)) break;
     }
     return up;
@@ -449,21 +463,6 @@ __device__ __forceinline__ float powerlaw_uplus(float R, const Phys &p)
     return R <= p.law_r2 ? r2 : p.pw_a * sqrtf(sqrtf(r2));
 }
 
-// One Newton step of Spalding's law for a lane: u+ and whether it has stopped.
-__device__ __forceinline__ void spalding_step(float R, const Phys &p, float &up, bool &done)
-{
-    const float k = p.kappa * up;
-    const float ek = expf(k);
-    const float k2 = __fmul_rn(k, k);
-    const float t2 = __fsub_rn(__fsub_rn(__fsub_rn(ek, 1.f), k), __fmul_rn(0.5f, k2));   // e^k - 1 - k - k^2/2
-    const float t3 = __fsub_rn(t2, __fmul_rn(__fmul_rn(k2, k), 1.f / 6.f));            // ... - k^3/6
-    const float S = __fmaf_rn(p.ekb, t3, up);                                           // y+(u+)
-    const float dS = __fmaf_rn(__fmul_rn(p.ekb, p.kappa), t2, 1.f);                     // dy+/du+
-    const float step = done ? 0.f : div_cell<false>(__fmaf_rn(up, S, -R), __fmaf_rn(up, dS, S));
-    up -= step;
-    done = done || fabsf(step) <= 1e-7f * up;
-}
-
 // u+ of the selected wall function (p.law is uniform over the launch).
 __device__ __forceinline__ float wall_uplus(float R, const Phys &p, unsigned mask)
 {
@@ -477,9 +476,7 @@ __device__ __forceinline__ float2 wall_uplus2(float2 R, const Phys &p, unsigned 
 {
     if (p.law == LAW_LOG) return make_float2(loglaw_uplus(R.x, p, mask), loglaw_uplus(R.y, p, mask));
     if (p.law == LAW_POWER) return make_float2(powerlaw_uplus(R.x, p), powerlaw_uplus(R.y, p));
-    float2 up = make_float2(sqrtf(R.x), sqrtf(R.y));
-    if (R.x > 100.f) up.x = fminf(up.x, __fadd_rn(logf(R.x) / p.kappa, p.B));
-    if (R.y > 100.f) up.y = fminf(up.y, __fadd_rn(logf(R.y) / p.kappa, p.B));
+    float2 up = make_float2(spalding_start(R.x, p), spalding_start(R.y, p));
     bool d0 = false, d1 = false;
     for (int it = 0; it < p.newton_iters; ++it) {
         spalding_step(R.x, p, up.x, d0);

@@ -184,41 +184,31 @@ __device__ __forceinline__ CellState collide(const float (&f)[Q], float (&fs)[Q]
 // feeds it (Eqs. 15-17): |tau_w| = rho (|u_t| / u+)^2 against u_t. The lanes
 // in `lanes` iterate the wall law together. Roundings are explicit here and in
 // the wall laws, so every kernel form computes the same tau_w.
-__device__ __forceinline__ void wfb_stress(const CellState &c, const Phys &p, unsigned lanes, float &twx, float &twz)
+__device__ __forceinline__ float wall_speed(const CellState &c) { return sqrtf(__fmaf_rn(c.uz, c.uz, __fmul_rn(c.ux, c.ux))); }
+__device__ __forceinline__ float wall_argument(float ut, const Phys &p) { return fmaxf(p.y1_over_nu * ut, 1e-30f); }
+
+__device__ __forceinline__ void wall_traction(const CellState &c, float ut, float up, float &twx, float &twz)
 {
-    twx = 0.f;
-    twz = 0.f;
-    const float ut = sqrtf(__fmaf_rn(c.uz, c.uz, __fmul_rn(c.ux, c.ux)));
-    const float R = fmaxf(p.y1_over_nu * ut, 1e-30f);
-    const float up = wall_uplus(R, p, lanes);
     const float utau = ut / up;
     const float tw = c.rho * utau * utau;
-    if (ut > 0.f) {
-        twx = -c.ux / ut * tw;
-        twz = -c.uz / ut * tw;
-    }
+    twx = ut > 0.f ? -c.ux / ut * tw : 0.f;
+    twz = ut > 0.f ? -c.uz / ut * tw : 0.f;
+}
+
+__device__ __forceinline__ void wfb_stress(const CellState &c, const Phys &p, unsigned lanes, float &twx, float &twz)
+{
+    const float ut = wall_speed(c);
+    wall_traction(c, ut, wall_uplus(wall_argument(ut, p), p, lanes), twx, twz);
 }
 
 // wfb_stress for two cells of a thread (c and b), their wall laws solved together.
 __device__ __forceinline__ void wfb_stress2(const CellState &c, const CellState &b, const Phys &p, float2 &twx,
                                             float2 &twz)
 {
-    twx = make_float2(0.f, 0.f);
-    twz = make_float2(0.f, 0.f);
-    const float ut = sqrtf(__fmaf_rn(c.uz, c.uz, __fmul_rn(c.ux, c.ux)));
-    const float vt = sqrtf(__fmaf_rn(b.uz, b.uz, __fmul_rn(b.ux, b.ux)));
-    const float2 up = wall_uplus2(make_float2(fmaxf(p.y1_over_nu * ut, 1e-30f), fmaxf(p.y1_over_nu * vt, 1e-30f)), p,
-                                  0xffffffffu);
-    const float us = ut / up.x, vs = vt / up.y;
-    const float tu = c.rho * us * us, tv = b.rho * vs * vs;
-    if (ut > 0.f) {
-        twx.x = -c.ux / ut * tu;
-        twz.x = -c.uz / ut * tu;
-    }
-    if (vt > 0.f) {
-        twx.y = -b.ux / vt * tv;
-        twz.y = -b.uz / vt * tv;
-    }
+    const float ut = wall_speed(c), vt = wall_speed(b);
+    const float2 up = wall_uplus2(make_float2(wall_argument(ut, p), wall_argument(vt, p)), p, 0xffffffffu);
+    wall_traction(c, ut, up.x, twx.x, twz.x);
+    wall_traction(b, vt, up.y, twx.y, twz.y);
 }
 
 // Full-way WFB at a wall node (layer 0 or ny - 1, WALL_NODE): f holds the
