@@ -134,8 +134,8 @@ typedef enum {
 } lbm_layout;
 
 /* Form of the fused step kernel (all compute the same update).
- *   CELL: one thread per cell, any grid (plain steps on odd nx with halfway walls
- *         and at least 2^17 cells run two cells per thread, the same bits).
+ *   CELL: one thread per cell, any grid (plain steps on large grids of odd nx with
+ *         halfway walls run two cells per thread, the same bits).
  *   PAIR: two cells per thread, 2-wide loads and packed FP32 math; even nx.
  *   TMA:  two cells per thread; each CTA streams whole source rows into a
  *         shared-memory ring with bulk asynchronous copies (full/empty

@@ -86,8 +86,9 @@ int select_kernel(lbm_handle *h, int kernel)
     h->kernel = kernel;
     const int per_row = h->g.nx / cells_per_thread(kernel);
     h->bx = row_threads(per_row);
-    // four-cell rows of just under four warps: two CTAs of two (448 cells: 43.3 us
-    // against 43.9)
+    // four-cell rows of just under four warps: two CTAs of two (us a step with one CTA
+    // / two, two-lattice BGK of nx x64x104: 388 cells 44.0 / 43.6, 416 43.6 / 43.1, 448
+    // 43.8 / 43.3, 480 45.1 / 44.6, 508 46.6 / 46.3; MRT and AA 0.1 to 0.6% less)
     if (kernel == LBM_KERNEL_QUAD && h->bx == 128 && per_row < 128) h->bx = 64;
     // Steps from lattice (or phase) 1 walk the planes backwards, so that each
     // step begins with the planes the step before wrote last, which L2 still
@@ -240,23 +241,40 @@ int configure_rows(lbm_handle *h)
 // FP32 64x32x32 5.4 / 5.4, 128x48x96 14.7 / 12.3, 256x64x128 52.4 / 50.2, AA 55.0 /
 // 51.9; FP16 MRT 256x64x128 37.3 / 32.4, 512x128x256 235.6 / 227.8, AA 256x64x128
 // 30.2 / 27.7, 64x32x32 8.6 / 5.4. The two-lattice FP32 step, bound by DRAM alone,
-// gains nothing at 512x128x256 (375.5 / 376.6) and loses 0.9% at 1024x256x512 (2961
-// / 2987), and at 64x32x32 it gains less than the larger graph costs to build, so
-// it is split between 2^18 and 2^25 cells; FP32 AA from 2^16 (16x8x8: 20 steps 105
-// us whole, 113 split).
+// gains nothing at 512x128x256 (375.5 / 376.6; MRT 395.4 / 394.6) and loses 0.9% at
+// 1024x256x512 (2961 / 2987; MRT 3131 / 3143), and at 64x32x32 it gains less than the
+// larger graph costs to build, so it is split between 2^18 and 2^25 cells; FP32 AA
+// from 2^16 (16x8x8: 20 steps 105 us whole, 113 split).
 constexpr long long kSplitFp32Min = 1LL << 18, kSplitFp32Max = 1LL << 25, kSplitFp32AaMin = 1LL << 16;
 // The even AA step of the four-cell kernel is better in one launch on large
 // grids (512x128x256 step pair: 208.1 against 214.1 us a step), on small ones not
 // (256x64x128: 27.7 against 27.1, 128x48x96: 11.1 against 10.0).
 constexpr long long kWholeEvenCells = 1LL << 23;
 
+// Warps that the CTAs of a row of per_row threads' work launch.
+int row_warps(int per_row)
+{
+    const int bx = row_threads(per_row);
+    return (per_row + bx - 1) / bx * (bx / 32);
+}
+
 // Whether plain steps of the one-cell form run two cells a thread (lbm_odd.cuh).
-// Below 2^17 cells the one-cell kernel's twice as many threads hide latency
-// better (99x20x28 FP32 6.3 us a step against 8.3; 125x20x131 13.5 against 11.4).
+// They pay by the warps they save a row: none below 33 cells, a third at 65 to 95,
+// half mostly. On small grids the one-cell kernel's more threads hide latency better.
+// us a step, one cell a thread / two: FP32 17x128x256 40.6 / 43.2, AA 29x256x256 75.4 /
+// 101; 95x58x56 FP32 10.2 / 10.5, AA 10.4 / 12.1, FP16 AA 10.6 / 12.2; 95x128x100 FP32
+// AA 37.5 / 50; 97x48x40 FP32 8.5 / 8.7, AA 8.7 / 9.4; 99x64x64 FP32 14.8 / 12.8, AA
+// 15.0 / 14.6, FP16 15.2 / 12.2. FP16 on two lattices gains from 2^17 cells and with a
+// third of the warps saved (65x50x56 1.03 times, 95x128x256 1.08), FP32 on two lattices
+// with a third from 2^20 (287x80x80 1.05 times, 95x128x256 1.11).
 bool odd_step(const lbm_handle *h)
 {
-    return h->kernel == LBM_KERNEL_CELL && h->g.nx % 2 == 1 && h->p.wall != lbm::WALL_NODE &&
-           (long long)h->g.nx * h->g.ny * h->g.nz >= 1LL << 17;
+    if (h->kernel != LBM_KERNEL_CELL || h->g.nx % 2 == 0 || h->p.wall == lbm::WALL_NODE) return false;
+    const long long cells = (long long)h->g.nx * h->g.ny * h->g.nz;
+    const int one = row_warps(h->g.nx), two = row_warps((h->g.nx + 1) / 2);
+    if (h->precision == LBM_FP16_SHIFTED && h->layout == LBM_PULL2) return one > two && cells >= 1LL << 17;
+    if (2 * one > 3 * two) return cells >= 1LL << 18;
+    return one > two && h->layout == LBM_PULL2 && cells >= 1LL << 20;
 }
 
 bool split_step(const lbm_handle *h)

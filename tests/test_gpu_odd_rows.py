@@ -33,3 +33,13 @@ def test_odd_rows_match_the_one_cell_kernel(nx, ny, nz, wall, precision, layout,
         ch.close()
     for a, b in zip(*out):
         assert np.array_equal(a, b)
+
+
+@pytest.mark.parametrize("mrt", [False, True])
+@pytest.mark.parametrize("layout", [lbm.PULL2, lbm.AA])
+@pytest.mark.parametrize("precision", [lbm.FP32, lbm.FP16_SHIFTED])
+@pytest.mark.parametrize("nx,ny,nz,wall", [  # both sides of 2^18 cells, and of 2^20 for rows of three warps against two
+    (33, 3, 2700, 1), (61, 2, 2200, 0), (63, 65, 64, 2), (63, 66, 64, 1), (127, 48, 43, 1), (129, 48, 48, 0), (257, 32, 33, 1),
+    (67, 126, 124, 1), (67, 128, 124, 1)])
+def test_odd_rows_of_larger_grids(nx, ny, nz, wall, precision, layout, mrt):
+    test_odd_rows_match_the_one_cell_kernel(nx, ny, nz, wall, precision, layout, mrt)
