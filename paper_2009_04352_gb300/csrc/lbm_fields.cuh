@@ -5,19 +5,22 @@
 // does, so DRAM bounds them as long as the rest stays small. The one-cell gather
 // of k_export with FP64 sums did not: FP64 runs at 1/64 of the FP32 rate here, and
 // FP16 storage was read 2 bytes at a time. us a call at 512x128x256, before / now
-// (floor, the reads and writes at the copy rate): conservation FP32 3980 / 388 (188),
-// AA 302, FP16 3967 / 300 (94), AA 229; plane profile FP32 739 / 320, AA 721 / 241 (188),
-// FP16 736 / 282 (94), AA 208; moments FP32 234 / 220 (228: a pass that mostly reads
+// (floor, the reads and writes at the copy rate): conservation FP32 3980 / 367 (188),
+// AA 277, FP16 3967 / 289 (94), AA 225; plane profile FP32 739 / 326, AA 721 / 219 (188),
+// FP16 736 / 261 (94), AA 204; moments FP32 234 / 220 (228: a pass that mostly reads
 // can beat the copy rate), FP16 206 / 158, AA 181 / 133 (134).
 // Here a thread gathers V cells of a row with the wide loads of the step kernels
 // (gather_pair, gather_quad), and the sums run in FP32 without loss against FP64:
 // every addition is an error-free transformation (Knuth's two-sum; products with
 // their FMA residual), its error is added to a second word error-free, and only the
 // errors of those additions to a third, with rounding. After n <= SUM_RUN cells the
-// three words move to FP64. With M the largest partial sum the second word stays
-// below 2 n 2^-24 M, the third below (2 n)^2 2^-48 M, so its roundings add up to less
-// than (2 n)^3 2^-72 M (2^-48 M for 128 cells, half the terms where a cell adds no
-// product); n additions in FP64 may lose n 2^-53 M, 2^-46 M.
+// three words are renormalised. With M the largest partial sum the second word stays
+// below 2 n 2^-24 M, the third below (2 n)^2 2^-48 M, so its roundings in a run add up
+// to less than (2 n)^3 2^-72 M (2^-48 M for 128 cells, an eighth where a cell adds no
+// product); n additions in FP64 may lose n 2^-53 M, 2^-46 M. Lanes and warps add their
+// words the same way, so that a block spends some thirty FP64 instructions: with the
+// words of every thread moved to FP64 it spent 165 a warp, 105 us of a call, which small
+// grids paid in full (conservation of 256x64x128 FP32 175 us, now 105; profile 90, now 64).
 #pragma once
 
 #include <algorithm>
@@ -27,7 +30,7 @@
 
 namespace lbm {
 
-constexpr int SUM_RUN = 128;   // cells in one compensated sum before it goes to FP64
+constexpr int SUM_RUN = 128;   // cells added to one sum before it is renormalised
 
 // a + b = s + e exactly, in both lanes.
 __device__ __forceinline__ float2 two_sum(float2 a, float2 b, float2 &e)
@@ -65,13 +68,61 @@ __device__ __forceinline__ void sum_mul(Sum3 &s, float2 a, float2 b)
     sum_add(s, v);
 }
 
-// Both sums in FP64; clears s.
-__device__ __forceinline__ double2 sum_take(Sum3 &s)
+// The same sums with mid no more than an ulp of hi and lo of mid, exactly.
+__device__ __forceinline__ void sum_renormalise(Sum3 &s)
 {
-    const double2 v = make_double2((double)s.hi.x + ((double)s.mid.x + (double)s.lo.x),
-                                   (double)s.hi.y + ((double)s.mid.y + (double)s.lo.y));
-    s.hi = s.mid = s.lo = bc(0.f);
-    return v;
+    float2 e;
+    s.hi = two_sum(s.hi, s.mid, e);
+    s.mid = two_sum(e, s.lo, s.lo);
+}
+
+// s += o
+__device__ __forceinline__ void sum_merge(Sum3 &s, const Sum3 &o)
+{
+    float2 e;
+    s.hi = two_sum(s.hi, o.hi, e);
+    sum_residual(s, e);
+    sum_residual(s, o.mid);
+    s.lo = add2(s.lo, o.lo);
+}
+
+// Both sums in FP64.
+__device__ __forceinline__ double2 sum_value(const Sum3 &s)
+{
+    return make_double2((double)s.hi.x + ((double)s.mid.x + (double)s.lo.x),
+                        (double)s.hi.y + ((double)s.mid.y + (double)s.lo.y));
+}
+
+__device__ __forceinline__ float2 shfl_xor2(float2 v, int o)
+{
+    return make_float2(__shfl_xor_sync(0xffffffffu, v.x, o), __shfl_xor_sync(0xffffffffu, v.y, o));
+}
+
+// Sum N Sum3 over the warp by reduce-scatter: lane l returns sum l / (32 / P) in
+// s[0], P the power of two from N up (lanes beyond sum N - 1 return others' copies).
+template <int N>
+__device__ __forceinline__ void warp_sums(Sum3 (&s)[N], int lane)
+{
+    constexpr int P = N > 8 ? 16 : 8;
+    static_assert(N > 4 && N <= 16, "six sums of a profile, ten of the directions");
+#pragma unroll
+    for (int h = P / 2, o = 16; o >= 1; h >>= 1, o >>= 1) {
+        const bool up = (lane & o) != 0;
+#pragma unroll
+        for (int i = 0; i < (h ? h : 1); ++i) {
+            Sum3 send = s[i], keep = s[i];
+            if (h && i + h < N) {
+                send.hi = up ? s[i].hi : s[i + h].hi, keep.hi = up ? s[i + h].hi : s[i].hi;
+                send.mid = up ? s[i].mid : s[i + h].mid, keep.mid = up ? s[i + h].mid : s[i].mid;
+                send.lo = up ? s[i].lo : s[i + h].lo, keep.lo = up ? s[i + h].lo : s[i].lo;
+            }
+            send.hi = shfl_xor2(send.hi, o);
+            send.mid = shfl_xor2(send.mid, o);
+            send.lo = shfl_xor2(send.lo, o);
+            sum_merge(keep, send);
+            s[i] = keep;
+        }
+    }
 }
 
 // f(t) of V cells as gathered: packed pairs, or for V = 4 the raw words of two
@@ -203,32 +254,6 @@ __global__ void __launch_bounds__(128) k_moments(const T *__restrict__ src, Geom
     }
 }
 
-// Sum N <= 16 doubles over the block by reduce-scatter (warp_stats_reduce of
-// lbm_kernels.cuh in FP64: 16 additions a lane instead of 5 N), then over the
-// warps in order; thread k < N returns sum k in v[0]. All threads must call it.
-template <int N>
-__device__ __forceinline__ double block_sums(double (&v)[16])
-{
-    __shared__ double red[4][16];
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-#pragma unroll
-    for (int h = 8, o = 16; h >= 1; h >>= 1, o >>= 1) {
-        const bool up = (lane & o) != 0;
-#pragma unroll
-        for (int i = 0; i < h; ++i) {
-            const double send = up ? v[i] : v[i + h], keep = up ? v[i + h] : v[i];
-            v[i] = keep + __shfl_xor_sync(0xffffffffu, send, o);
-        }
-    }
-    const double w = v[0] + __shfl_xor_sync(0xffffffffu, v[0], 1);
-    if (!(lane & 1)) red[warp][lane >> 1] = w;
-    __syncthreads();
-    double s = 0.0;
-    if (threadIdx.x < N)
-        for (int i = 0; i < (int)(blockDim.x >> 5); ++i) s += red[i][threadIdx.x];
-    return s;
-}
-
 constexpr float VEL_SCALE = 1073741824.f;   // 2^30
 
 // Whether a cell's terms go to the FP32 sums: rho from 1/2, below which rho - 1
@@ -241,23 +266,15 @@ __device__ __forceinline__ bool profile_in_range(float rho, float ux, float uy, 
     const float ax = fabsf(ux), ay = fabsf(uy), az = fabsf(uz);
     // 0 wraps round to the largest word
     const unsigned least = min(__float_as_uint(ax) - 1u, min(__float_as_uint(ay) - 1u, __float_as_uint(az) - 1u));
-    return rho >= 0.5f && rho <= 16777216.f && ax + ay + az < 1e6f && least >= ((127u - 81u) << 23) - 1u;
+    return rho >= 0.5f && rho <= 16777216.f && ax + ay + az < 65536.f && least >= ((127u - 81u) << 23) - 1u;
 }
 
-__device__ __forceinline__ void profile_add_fp64(double (&v)[16], float rho, float fx, float fy, float fz)
+__device__ __forceinline__ void profile_add_fp64(double (*v)[128], float rho, float fx, float fy, float fz)
 {
     const double r = rho, ux = fx, uy = fy, uz = fz;
-    v[0] += r;
-    v[1] += ux;
-    v[2] += uy;
-    v[3] += uz;
-    v[4] += ux * ux;
-    v[5] += uy * uy;
-    v[6] += uz * uz;
-    v[7] += ux * uy;
-    v[8] += r * ux;
-    v[9] += r * uy;
-    v[10] += r * uz;
+    const double t[K_STATS] = {r, ux, uy, uz, ux * ux, uy * uy, uz * uz, ux * uy, r * ux, r * uy, r * uz};
+#pragma unroll
+    for (int k = 0; k < K_STATS; ++k) v[k][threadIdx.x] += t[k];
 }
 
 // Sums over the row tiles blockIdx.x, blockIdx.x + gridDim.x, ... of plane
@@ -269,50 +286,29 @@ __device__ __forceinline__ void profile_add_fp64(double (&v)[16], float rho, flo
 // (or opposite directions) of one cell, not one column of two cells: half the
 // registers for the same packed additions. The order of the additions depends on the
 // grid only, so every layout and storage map gives the same bits.
-// CTAs per SM the register budget must allow (us at 512x128x256 with sixteen CTAs an
-// SM in all, 3 / 4 / 5 / 6): FP32 profile 388 / 412 / 337 / 362, AA 232 / 235 / 258 /
-// 253, conservation 450 / 459 / 415 / 573, AA 315 / 294 / 328 / 450; FP16 profile 278 /
-// 283 / 300 / 304, conservation 302 / 299 / 340 / 400.
-template <typename T, int LAY> constexpr int SUM_BLOCKS = sizeof(T) == 4 && LAY == LAY_PULL ? 5 : 4;
+// CTAs per SM the register budget must allow (us at 512x128x256, 4 / 5): FP32 profile
+// 326 / 366, AA 231 / 219, conservation 466 / 367, AA 278 / 290; FP16 profile 262 / 270,
+// AA 205 / 210, conservation 291 / 302, AA 226 / 250; 6 is slower than both.
+template <typename T, int LAY, bool PROFILE> constexpr int SUM_BLOCKS = sizeof(T) == 4 && PROFILE != (LAY == LAY_PULL) ? 5 : 4;
 
 template <typename T, int V, int LAY, bool PROFILE>
-__global__ void __launch_bounds__(128, SUM_BLOCKS<T, LAY>) k_plane_sums(const T *__restrict__ src, Geom g, Phys p, int nxb,
+__global__ void __launch_bounds__(128, SUM_BLOCKS<T, LAY, PROFILE>) k_plane_sums(const T *__restrict__ src, Geom g, Phys p, int nxb,
                                                                          double *__restrict__ out)
 {
     constexpr int NP = (V + 1) / 2, NS = PROFILE ? (K_STATS + 1) / 2 : (Q + 1) / 2, NOUT = PROFILE ? K_STATS : 4;
-    const int lane = threadIdx.x & 31, y = blockIdx.y;
+    __shared__ Sum3 red[4][NS];
+    __shared__ int count[4];
+    __shared__ double beyond[PROFILE ? K_STATS : 1][128];   // terms that FP32 does not hold, a column a thread
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, y = blockIdx.y;
     const int tiles = nxb * g.nz;
     Sum3 s[NS];
 #pragma unroll
     for (int k = 0; k < NS; ++k) s[k].hi = s[k].mid = s[k].lo = bc(0.f);
-    double v[16];
+    if (PROFILE) {
 #pragma unroll
-    for (int k = 0; k < 16; ++k) v[k] = 0.0;
-    auto take = [&]() {
-        if constexpr (PROFILE) {
-            const double s1 = 1.0 / (double)VEL_SCALE, s2 = s1 * s1;
-#pragma unroll
-            for (int k = 0; k < NS; ++k) {
-                const double2 t = sum_take(s[k]);
-                const double scale = k < 2 ? 1.0 : (k < 4 ? s2 : s1);
-                v[2 * k] += t.x * scale;
-                if (2 * k + 1 < K_STATS) v[2 * k + 1] += t.y * scale;
-            }
-        } else {
-            const double2 rest = sum_take(s[9]);
-            v[0] += rest.x + rest.y;
-#pragma unroll
-            for (int k = 0; k < 9; ++k) {
-                const int a = 2 * k + 1;
-                const double2 t = sum_take(s[k]);
-                const double d = t.x - t.y;
-                v[0] += t.x + t.y;
-                if (ex_of(a)) v[1] += ex_of(a) > 0 ? d : -d;
-                if (ey_of(a)) v[2] += ey_of(a) > 0 ? d : -d;
-                if (ez_of(a)) v[3] += ez_of(a) > 0 ? d : -d;
-            }
-        }
-    };
+        for (int k = 0; k < K_STATS; ++k) beyond[k][threadIdx.x] = 0.0;
+    }
+    bool fp64 = false;
     int run = 0, cells = 0;
     for (int t = blockIdx.x; t < tiles; t += gridDim.x) {
         const int z = t / nxb, x0 = V * ((t - z * nxb) * blockDim.x + threadIdx.x);
@@ -342,7 +338,8 @@ __global__ void __launch_bounds__(128, SUM_BLOCKS<T, LAY>) k_plane_sums(const T 
                             sum_mul(s[4], bc(rho), vxy);
                             sum_mul(s[5], make_float2(rho, 0.f), make_float2(vz, 0.f));
                         } else {
-                            profile_add_fp64(v, rho, ux, uy, uz);
+                            profile_add_fp64(beyond, rho, ux, uy, uz);
+                            fp64 = true;
                         }
                     }
                 } else {
@@ -357,14 +354,52 @@ __global__ void __launch_bounds__(128, SUM_BLOCKS<T, LAY>) k_plane_sums(const T 
         }
         run += V;
         if (run + V > SUM_RUN) {
-            take();
+#pragma unroll
+            for (int k = 0; k < NS; ++k) sum_renormalise(s[k]);
             run = 0;
         }
     }
-    take();
-    if (PROFILE) v[0] += (double)cells;
-    const double r = block_sums<NOUT>(v);
-    if (threadIdx.x < NOUT) out[((long long)y * gridDim.x + blockIdx.x) * NOUT + threadIdx.x] = r;
+    warp_sums<NS>(s, lane);
+    constexpr int LANES = NS > 8 ? 2 : 4;   // lanes that return a sum
+    if (lane % LANES == 0 && lane / LANES < NS) red[warp][lane / LANES] = s[0];
+    if (PROFILE) {
+        const int c = __reduce_add_sync(0xffffffffu, cells);
+        if (lane == 0) count[warp] = c;
+    }
+    fp64 = __syncthreads_or(fp64);
+    if (warp != 0) return;
+    const int warps = blockDim.x >> 5;
+    Sum3 t = red[0][min(lane, NS - 1)];
+    for (int w = 1; w < warps; ++w) sum_merge(t, red[w][min(lane, NS - 1)]);
+    double2 v = sum_value(t);
+    out += ((long long)y * gridDim.x + blockIdx.x) * NOUT;
+    if constexpr (PROFILE) {
+        if (lane >= NS) return;
+        const bool last = 2 * lane + 1 >= K_STATS;
+        if (lane > 1) {
+            const double scale = 1.0 / (double)VEL_SCALE * (lane < 4 ? 1.0 / (double)VEL_SCALE : 1.0);
+            v = make_double2(v.x * scale, v.y * scale);
+        }
+        if (lane == 0)
+            for (int w = 0; w < warps; ++w) v.x += (double)count[w];
+        if (fp64)
+            for (int i = 0; i < (int)blockDim.x; ++i) {
+                v.x += beyond[2 * lane][i];
+                if (!last) v.y += beyond[2 * lane + 1][i];
+            }
+        out[2 * lane] = v.x;
+        if (!last) out[2 * lane + 1] = v.y;
+    } else {
+        // sums 0 .. 8 hold directions a = 2 k + 1 and a + 1 = opp(a), sum 9 the rest population of both cells
+        const int a = lane < 9 ? 2 * lane + 1 : 0;
+        const double d = v.x - v.y;
+        double r[4] = {lane < NS ? v.x + v.y : 0.0, ex_of(a) * d, ey_of(a) * d, ez_of(a) * d};
+#pragma unroll
+        for (int o = 8; o >= 1; o >>= 1)
+#pragma unroll
+            for (int k = 0; k < 4; ++k) r[k] += __shfl_xor_sync(0xffffffffu, r[k], o);
+        if (lane < 4) out[lane] = lane == 0 ? r[0] : (lane == 1 ? r[1] : (lane == 2 ? r[2] : r[3]));
+    }
 }
 
 // Cells a thread gathers at once on rows of nx cells.
@@ -374,12 +409,11 @@ inline int cells_wide(const lbm_handle *h)
 }
 
 // CTAs of k_plane_sums for each plane: five rounds of the four CTAs an SM holds of
-// the 152 of this GPU over all planes (four of the five in two-lattice FP32), at most
-// one for each row tile and `most`. The number of SMs is written out, as the order of
-// the additions must not depend on the device. us at 512x128x256 with one / two /
-// three / four rounds of five: FP32 profile 439 / 352 / 327 / 320, conservation 529 /
-// 401 / 391 / 388; of four: FP16 profile 369 / 303 / 286 / 281, conservation 402 / 306 /
-// 297 / 296.
+// the 152 of this GPU over all planes, at most one for each row tile and `most`. The
+// number of SMs is written out, as the order of the additions must not depend on the
+// device. us with 16 / 20 / 24 / 30 CTAs an SM, FP32 on two lattices: 512x128x256 profile
+// 335 / 326 / 318 / 313, conservation 388 / 365 / 359 / 362; 446x16x157 43 / 44 / 48 / 50
+// and 91 / 93 / 89 / 99; 256x64x128 63 / 64 / 66 / 66 and 106 / 105 / 112 / 114.
 inline int plane_sum_blocks(const lbm_handle *h, int most)
 {
     const int v = cells_wide(h), per_row = h->g.nx / v, bx = row_threads(per_row);

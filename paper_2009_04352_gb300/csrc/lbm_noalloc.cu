@@ -51,15 +51,27 @@ int scratch_on_current_device(double **out)
     return LBM_OK;
 }
 
-// The partials of each plane (k_plane_sums of lbm_fields.cuh) in order.
-__global__ void k_profile_finish(const double *__restrict__ scratch, int ny, int blocks, double *__restrict__ out)
+// The partials of each plane (k_plane_sums of lbm_fields.cuh) in fixed order, one block
+// of 256 a plane: sixteen groups of threads share the partials, a column a thread (few
+// planes have hundreds of partials each; added by one thread they took 40 us of a
+// call at 291x13x65).
+__global__ void __launch_bounds__(256) k_profile_finish(const double *__restrict__ scratch, int blocks, double *__restrict__ out)
 {
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= ny * lbm::K_STATS) return;
-    const int y = i / lbm::K_STATS, k = i % lbm::K_STATS;
+    __shared__ double red[16][16];
+    const int y = blockIdx.x, k = threadIdx.x & 15, grp = threadIdx.x >> 4;
+    double v = 0.0;
+    if (k < lbm::K_STATS) {
+        const double *q = scratch + (long long)y * blocks * lbm::K_STATS + k;
+#pragma unroll 4
+        for (int b = grp; b < blocks; b += 16) v += q[b * lbm::K_STATS];
+    }
+    red[grp][k] = v;
+    __syncthreads();
+    if (threadIdx.x >= lbm::K_STATS) return;
     double s = 0.0;
-    for (int b = 0; b < blocks; ++b) s += scratch[((long long)y * blocks + b) * lbm::K_STATS + k];
-    out[i] = s;
+#pragma unroll
+    for (int i = 0; i < 16; ++i) s += red[i][k];
+    out[y * lbm::K_STATS + k] = s;
 }
 
 }  // namespace
@@ -78,8 +90,7 @@ extern "C" int lbm_plane_profile_noalloc(lbm_handle *h, double *out_dev)
     lbm::plane_sums<true>(h, blocks, scratch);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return lbm_record_error(LBM_ERR_CUDA, cudaGetErrorString(e));
-    const int n = h->g.ny * lbm::K_STATS;
-    k_profile_finish<<<(n + 127) / 128, 128, 0, h->stream>>>(scratch, h->g.ny, blocks, out_dev);
+    k_profile_finish<<<h->g.ny, 256, 0, h->stream>>>(scratch, blocks, out_dev);
     e = cudaGetLastError();
     if (e != cudaSuccess) return lbm_record_error(LBM_ERR_CUDA, cudaGetErrorString(e));
     return LBM_OK;
