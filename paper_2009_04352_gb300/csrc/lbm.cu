@@ -244,8 +244,10 @@ int configure_rows(lbm_handle *h)
 // gains nothing at 512x128x256 (375.5 / 376.6; MRT 395.4 / 394.6) and loses 0.9% at
 // 1024x256x512 (2961 / 2987; MRT 3131 / 3143), and at 64x32x32 it gains less than the
 // larger graph costs to build, so it is split between 2^18 and 2^25 cells; FP32 AA
-// from 2^16 (16x8x8: 20 steps 105 us whole, 113 split).
-constexpr long long kSplitFp32Min = 1LL << 18, kSplitFp32Max = 1LL << 25, kSplitFp32AaMin = 1LL << 16;
+// from 2^16 (16x8x8: 20 steps 105 us whole, 113 split), and so are the two cells a
+// thread of FP16 (64 steps, whole / split: 30x20x20 281 / 330, 62x40x20 323 / 350, AA 330 /
+// 350, MRT 323 / 333; 66x48x40 453 / 420, AA 471 / 429, MRT 471 / 413).
+constexpr long long kSplitFp32Min = 1LL << 18, kSplitFp32Max = 1LL << 25, kSplitMin = 1LL << 16;
 // The even AA step of the four-cell kernel is better in one launch on large
 // grids (512x128x256 step pair: 208.1 against 214.1 us a step), on small ones not
 // (256x64x128: 27.7 against 27.1, 128x48x96: 11.1 against 10.0).
@@ -281,8 +283,9 @@ bool split_step(const lbm_handle *h)
 {
     if (h->kernel == LBM_KERNEL_TMA || (h->kernel == LBM_KERNEL_CELL && !odd_step(h)) || h->g.ny < 3) return false;
     const long long cells = (long long)h->g.nx * h->g.ny * h->g.nz;
-    if (h->precision == LBM_FP16_SHIFTED) return true;
-    return h->layout == LBM_AA ? cells >= kSplitFp32AaMin : cells >= kSplitFp32Min && cells < kSplitFp32Max;
+    if (h->kernel == LBM_KERNEL_QUAD) return true;
+    if (h->precision == LBM_FP16_SHIFTED || h->layout == LBM_AA) return cells >= kSplitMin;
+    return cells >= kSplitFp32Min && cells < kSplitFp32Max;
 }
 
 // Whether a plain one-launch FP32 two-lattice step of the two-cell kernel on stream

@@ -14,7 +14,8 @@ pytestmark = pytest.mark.gpu
 CASES = [  # nx, ny, nz, precision, layout, collision, wall
     (64, 32, 32, lbm.FP32, lbm.PULL2, 0, 1), (63, 12, 14, lbm.FP32, lbm.AA, 0, 1),          # one launch a step
     (96, 48, 57, lbm.FP32, lbm.PULL2, 0, 1), (64, 32, 34, lbm.FP32, lbm.AA, 1, 1),          # two, planes forwards
-    (66, 12, 14, lbm.FP16_SHIFTED, lbm.PULL2, 0, 0), (64, 16, 16, lbm.FP16_SHIFTED, lbm.AA, 0, 1),
+    (66, 12, 14, lbm.FP16_SHIFTED, lbm.PULL2, 0, 0), (66, 40, 26, lbm.FP16_SHIFTED, lbm.AA, 0, 1),
+    (129, 40, 32, lbm.FP16_SHIFTED, lbm.PULL2, 1, 1), (64, 16, 16, lbm.FP16_SHIFTED, lbm.AA, 0, 1),
     (160, 64, 64, lbm.FP32, lbm.PULL2, 0, 1), (162, 64, 70, lbm.FP32, lbm.PULL2, 1, 3),     # planes in alternating order
     (161, 64, 72, lbm.FP32, lbm.PULL2, 0, 1), (160, 64, 130, lbm.FP32, lbm.AA, 0, 1),
     (256, 64, 82, lbm.FP16_SHIFTED, lbm.PULL2, 0, 1), (252, 65, 83, lbm.FP16_SHIFTED, lbm.PULL2, 1, 1),
