@@ -956,7 +956,7 @@ int lbm_step(lbm_handle *h, int n)
         if (rc != LBM_OK) return rc;
     }
     const int chunk = chunk_steps(h), period = period_steps(h);
-    const bool quarters = graphs && use_quarters(h);
+    const bool quarters = graphs && use_quarters(h), split = split_step(h);
     while (n > 0) {
         const bool sample = h->stats_every > 0 && (h->step % h->stats_every) == 0;
         if (graphs && sample && period > 1 && n >= period && h->period[h->cur].steps == period) {
@@ -981,12 +981,17 @@ int lbm_step(lbm_handle *h, int n)
             const long long to_next = h->stats_every - (h->step % h->stats_every);
             if (to_next < run) run = to_next;
         }
+        // 12 or 16 two-launch steps from phase 1 go in quarters alone: after a single step
+        // and a chunk three more single steps would be left (us for 16 steps of 64x32x32
+        // FP16 112 / 102, 256x32x32 129 / 117, FP32 AA 130x64x64 253 / 240). From 24 steps on the
+        // gaps between the quarters cost more (64 steps of 256x32x32: 424 / 460).
+        const bool whole = split && h->cur == 1 && run <= 2 * chunk && run % kQuarterSteps == 0;
         while (run > 0) {
             int done;
             if (graphs && h->cur == 0 && run >= chunk) {
                 done = chunk;
                 CK(cudaGraphLaunch(h->chunk.exec, h->stream));
-            } else if (quarters && run >= kQuarterSteps && run <= chunk) {
+            } else if (quarters && run >= kQuarterSteps && (run <= chunk || whole)) {
                 done = kQuarterSteps;
                 CK(cudaGraphLaunch(h->quarter[h->cur].exec, h->stream));
             } else {

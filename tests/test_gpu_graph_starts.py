@@ -42,7 +42,7 @@ def _run(case, precision, layout, mrt, every, chunks):
     return state.view(dtype).view(19, case.nz, case.ny, sx)[..., :case.nx], tau, sums
 
 
-@pytest.mark.parametrize("every,chunks", [(0, [16, 3, 6, 16]), (0, [1, 8, 24]), (6, [3, 33]), (7, [3, 40]), (7, [4, 1, 40])])
+@pytest.mark.parametrize("every,chunks", [(0, [16, 3, 6, 16]), (0, [1, 8, 24]), (0, [1, 12, 16]), (6, [3, 33]), (7, [3, 40]), (7, [4, 1, 40])])
 @pytest.mark.parametrize("nx,ny,nz,precision,layout,mrt,wall", CASES)
 def test_graphs_of_either_start(nx, ny, nz, precision, layout, mrt, wall, every, chunks):
     case = workload.derive_channel("starts", nx, ny, nz, 640.0, wall=wall)
