@@ -35,7 +35,7 @@ METRIC = "MLUPS and % of HBM roofline, FP32 vs FP16-storage vs batched, at state
 BYTES_PER_LUP = {0: 152, 1: 76}     # 19 reads + 19 writes, FP32 / FP16 storage
 FALLBACK_HBM_GBS = 6800.0
 NOMINAL_HBM_GBS = 7900.0      # GB300 HBM3e nominal, for the second fraction
-GRAPH_STEPS = 16              # steps per replayed CUDA graph in the library
+GRAPH_STEPS = 16              # a multiple of the steps of the library's plain graphs (4, 8 or 16)
 SAMPLE_CELLS = 2_100_000      # cells of the bounded oracle sample (a z-slab of the workload)
 
 # DRAM traffic per launch (dram__bytes_read.sum + dram__bytes_write.sum) of the
