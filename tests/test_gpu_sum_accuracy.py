@@ -58,7 +58,7 @@ def test_profile_of_uniform_planes(nx, precision, layout):
     ch = lbm.Channel.from_case(case, precision=precision, layout=layout)
     ch.init_channel(workload.u_mean_profile(case), 0.0, 3)
     ch.step(1)
-    # three additions for each of at most three sums of a thread, nine in the block, at most 30 blocks a plane
+    # three additions for the words of a block's sum, its share of the error-free runs, at most 30 blocks a plane
     _check_profile(ch, 48)
     ch.close()
 
@@ -97,8 +97,8 @@ def test_conservation_of_spread_magnitudes(nx, layout):
     ch.set_populations(np.broadcast_to(W + z[None, :, None, None], (19, nz, ny, nx)))
     fb = z.astype(np.float32).astype(np.float64) * (nx * ny)
     total = ch.conservation()
-    # at most three sums of a thread with three additions each, the 19 directions, nine additions in the block,
-    # ten blocks a thread and eight levels in the last reduction; the cells' rest mass is added last
+    # three additions for the words of a block's sums, the directions, ten blocks a thread and eight levels in the
+    # last reduction, and the error-free runs' share; the cells' rest mass is added last
     assert abs(total[0] - (19 * math.fsum(fb) + case.cells)) <= 64 * 2.0 ** -53 * 19 * math.fsum(fb) + 2.0 ** -52 * total[0]
     for k in range(3):
         assert abs(total[1 + k]) <= 64 * 2.0 ** -53 * 19 * math.fsum(fb)
